@@ -37,8 +37,10 @@ static const int kTimingEvents = 256;
 static const int kMaxParts = 320;      // most split-V records any kernel writes per row
 static const int kStreamMaxRows = 16;  // largest M the streaming path is chosen for
 static const int kSplitCodeRows = 256;  // tensor path: z carried as hi + lo bf16 parts while the call is HBM-bound (up to this many rows)
+static const int kTcK = 64;             // the tensor-core down-projection: d a multiple of this, r at least this
 static const int kRowPad = 8;          // rows of the generic path's fp32 code are padded to this
-static const int kStreamTile = 16;     // rows one launch of the streaming kernels takes
+static const int kStreamTile = 16;     // rows one launch of the older streaming kernels takes
+static const int kSlabRows = 64;       // rows one launch of the slab kernel takes
 static const int kCodeByStreamRows = 32;   // tensor path: up to this many rows z comes from the streaming path's down-projection
 
 static int round_up(int x, int m) { return (x + m - 1) / m * m; }
@@ -79,10 +81,10 @@ extern "C" int slimspec_create(slimspec_ctx** out, int max_M, int max_d, int max
     const size_t z_elems = mpad * (size_t)max_d;
     // split-V records, padded to 16 bytes: the streaming path writes <= 16 rows x 320 records, the
     // tensor path 128 * nrb rows x (SMs / nrb) slabs
-    const int rec_k = max_k < 32 ? max_k : 32;
+    const int rec_k = max_k;
     const size_t mpad128 = (size_t)round_up(max_M, 128);
     const size_t part_elems = ((size_t)kStreamTile * kMaxParts + (size_t)(c->sm_count + 12) * 256 + 2 * mpad128) *
-                              (size_t)round_up(2 + 2 * rec_k, 4);
+                              (size_t)(2 + 2 * rec_k);
     // K-split partial tiles of the tensor-core down-projection: one 128 x 128 fp32 tile per SM, or one split
     size_t zpart_elems = (size_t)(c->sm_count + 12) * 128 * 128;
     if (zpart_elems < mpad128 * (size_t)max_d) zpart_elems = mpad128 * (size_t)max_d;
@@ -117,7 +119,7 @@ extern "C" int slimspec_create(slimspec_ctx** out, int max_M, int max_d, int max
     ok = ok && cudaMemset(c->s.err, 0, sizeof(int)) == cudaSuccess;
     ok = ok && cudaMemset(c->s.zq, 0, fma_code_words(max_d) * sizeof(uint2)) == cudaSuccess;
     ok = ok && cudaMemset(c->s.z, 0, z_elems * sizeof(float)) == cudaSuccess;
-    ok = ok && stream_prepare() == cudaSuccess && fma_prepare() == cudaSuccess;
+    ok = ok && stream_prepare() == cudaSuccess && slab_prepare() == cudaSuccess && fma_prepare() == cudaSuccess;
     ok = ok && cudaDeviceSynchronize() == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -254,11 +256,16 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
     const bool ptr_ok = aligned16(h) && aligned16(Bm) && (!lowrank || aligned16(A)) &&
                         (mode == 0 || aligned16(logits));
     StreamPlan sp = stream_plan(M, K, V, mode == 0 ? k : 1, c->sm_count);
-    const bool stream_ok = sp.ok && ptr_ok && d % 2 == 0 && (!lowrank || r % 16 == 0);
-    const bool tensor_fits = tensor_ok(M, K, V, k, mode) && ptr_ok && (!lowrank || (d % 64 == 0 && r >= 64));
+    const int slab_rows = M < kSlabRows ? M : kSlabRows;
+    // (Raw logits of up to 16 rows have no selection to save and stay with the older kernels: M = 4, d = 2048,
+    // r = 256: 18.4 us there, 19.4 us here.)
+    const bool slab = ptr_ok && d % 2 == 0 && (!lowrank || r % 16 == 0) && slab_ok(slab_rows, lowrank, K, V, mode == 0 ? k : 1, c->sm_count) &&
+                      !(mode == 1 && M <= kStreamMaxRows && sp.ok);
+    const bool stream_ok = (slab && k <= 32) || (sp.ok && ptr_ok && d % 2 == 0 && (!lowrank || r % 16 == 0));
+    const bool tensor_fits = tensor_ok(M, K, V, k, mode) && ptr_ok && (!lowrank || (d % kTcK == 0 && r >= kTcK));
     if (path == SLIMSPEC_PATH_AUTO) {
         // FP32 FMAs keep up with HBM only for a few rows; beyond that the tensor cores take over
-        if (M > kStreamMaxRows && tensor_fits) path = SLIMSPEC_PATH_TENSOR;
+        if (M > (slab ? kSlabRows : kStreamMaxRows) && tensor_fits) path = SLIMSPEC_PATH_TENSOR;
         else path = stream_ok ? SLIMSPEC_PATH_STREAM : (tensor_fits ? SLIMSPEC_PATH_TENSOR : SLIMSPEC_PATH_GENERIC);
     }
     if (path == SLIMSPEC_PATH_TENSOR && !tensor_fits) return SLIMSPEC_ERR_ALIGN;
@@ -317,15 +324,22 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
     }
 
     // streaming path: row tiles of up to 16 rows, each streams the K x V matrix once
-    for (int m0 = 0; m0 < M; m0 += kStreamTile) {
-        const int mrows = (M - m0 < kStreamTile) ? (M - m0) : kStreamTile;
+    const int tile_rows = slab ? kSlabRows : kStreamTile;
+    for (int m0 = 0; m0 < M; m0 += tile_rows) {
+        const int mrows = (M - m0 < tile_rows) ? (M - m0) : tile_rows;
         const bf16* hm = h + (size_t)m0 * d;
         const int kk = mode == 0 ? k : 1;
         int nl = 0;
         // one or two rows: the FMA kernel, one launch; three to sixteen: the tensor-core streaming kernels
         const FmaPlan fp = fma_plan(mrows, d, lowrank ? r : 0, V, kk, c->sm_count);
         const bool fma = fp.ok && fp.ncta <= c->s.max_parts;
-        if (!fma) {
+        const bool use_slab = !fma && slab && slab_ok(mrows, lowrank, K, V, kk, c->sm_count);
+        if (use_slab) {
+            // the streaming path's down-projection reads A once per 16 rows: beyond 32 the K-split tensor-core product
+            // and its reduction are faster (64 rows, d = 8192, r = 1024: whole call 115.5 us with the one, 81.7 us with the other)
+            if (lowrank && mrows > kCodeByStreamRows && d % kTcK == 0 && r >= kTcK) CK(tensor_downproj(hm, A, mrows, d, r, true, c->s, c->sm_count, &nl, st));
+            else if (lowrank) { CK(stream_code_rows(hm, A, mrows, d, r, c->s.zb, c->s.zb_lo, c->sm_count, st)); nl = 1; }
+        } else if (!fma) {
             if (lowrank) CK(stream_code(hm, A, mrows, d, r, V, kk, c->s.zfrag, c->sm_count, st));
             else CK(stream_widen(hm, mrows, d, V, kk, c->s.zfrag, c->sm_count, st));
             nl = 1;
@@ -346,6 +360,10 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
                 c->epoch = 1;
             }
             CK(fma_head(hm, A, Bm, mrows, fp.mt, d, r, V, kk, mode, ids_t, lp_t, lg_t, c->s, c->epoch, c->sm_count, st));
+            nl += 1;
+        } else if (use_slab) {
+            CK(slab_head(lowrank ? c->s.zb : hm, lowrank ? c->s.zb_lo : (const bf16*)nullptr, Bm, mrows, K, V, kk, mode, ids_t, lp_t, lg_t, c->s,
+                         c->sm_count, slot < 0, st));
             nl += 1;
         } else {
             int nh = 0;

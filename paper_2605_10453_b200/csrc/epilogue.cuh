@@ -30,6 +30,52 @@ __device__ __forceinline__ unsigned int ld_acquire_gpu_u32(const unsigned int* p
 static constexpr long long kArrivalPolls = 1ll << 22;      // reads of the counter before a merging CTA gives up (seconds)
 
 // ------------------------------------------------------------------------------------------
+// Arrival and merge, by all threads of the CTA, when the CTA's records are written.  The CTAs take
+// tickets from a counter that only counts up (the call's first ticket is p.ticket_base).  The last R of
+// them to arrive merge: each takes every R-th row, waits until the counter shows that all P have arrived
+// (they are already running: it is a wait of a microsecond, bounded all the same), and runs two tasks per
+// row, a warp each: the row's log-sum-exp, and its k best entries.  s_ticket: a word of shared memory;
+// merge_area: merge_area_bytes(rows per merger, warps with a task) of it, 16-byte aligned.
+__host__ __device__ constexpr int merge_area_bytes(int rows, int warps) { return 64 + rows * kMaxK * 8 + warps * kMergeWarpBytes; }
+template <class Params>
+__device__ __forceinline__ void merge_by_last_arrivals(const Params& p, unsigned int* s_ticket, unsigned char* merge_area)
+{
+    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nt = blockDim.x, nw = nt >> 5;
+    const int k = p.k, P = p.ncta;
+    __syncthreads();
+    if (tid == 0) *s_ticket = ticket_take(p.ticket) - p.ticket_base;
+    __syncthreads();
+    const int rows_at_once = max(1, nw >> 1);
+    const int R = min(P, (p.M + rows_at_once - 1) / rows_at_once);
+    const int me = (int)*s_ticket - (P - R);             // which of the R mergers this CTA is
+    if (me < 0) return;
+    if (me != R - 1) {
+        if (tid == 0) {
+            long long it = 0;
+            while (ld_acquire_gpu_u32(p.ticket) - p.ticket_base < (unsigned)P && ++it < kArrivalPolls) {}
+            if (it >= kArrivalPolls) atomicCAS(p.err, 0, ERR_WAIT_RECORD);
+        }
+        __syncthreads();
+    }
+    const int mine = (p.M - me + R - 1) / R;             // rows me, me + R, ... (at most sixteen)
+    float* lse_s = reinterpret_cast<float*>(merge_area);                                         // [16]
+    unsigned long long* out = reinterpret_cast<unsigned long long*>(merge_area + 64);            // [mine][kMaxK] ordered entries
+    unsigned char* area = merge_area + 64 + mine * kMaxK * 8 + warp * kMergeWarpBytes;
+    for (int task = warp; task < 2 * mine; task += nw) {
+        const int lr = task >> 1, row = me + lr * R;
+        if (P <= 5 * 32) merge_task<5>(p.part, P, k, row, task & 1, lane, lse_s + lr, out + lr * kMaxK, area);
+        else merge_task<kMergeLists>(p.part, P, k, row, task & 1, lane, lse_s + lr, out + lr * kMaxK, area);
+    }
+    __syncthreads();
+    for (int e = tid; e < mine * k; e += nt) {
+        const int lr = e / k, j = e - lr * k, row = me + lr * R;
+        const unsigned long long c = out[lr * kMaxK + j];
+        p.ids[(size_t)row * k + j] = cand_id(c);
+        p.logprobs[(size_t)row * k + j] = key2f(cand_key(c)) - lse_s[lr];
+    }
+}
+
+// ------------------------------------------------------------------------------------------
 // Step (4) of the epilogue and what follows it: a warp per row orders the parked candidates by counting
 // and writes the slab's record; then the arrival ticket, and the last CTAs to arrive merge the records.
 template <int MT, class Params>
@@ -45,7 +91,7 @@ __device__ __forceinline__ void slab_records(const Params& p, unsigned char* sme
     uint32_t* ck = reinterpret_cast<uint32_t*>(scratch);      // [MT][kCand]
     int* ci = reinterpret_cast<int*>(ck + MT * kCand);
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nt = blockDim.x, nw = nt >> 5;
+    const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = blockDim.x >> 5;
     const int cta = blockIdx.x, k = p.k;
     const int mrows = min(p.M, MT);
     auto logit = [&](int row, int c) {
@@ -56,16 +102,15 @@ __device__ __forceinline__ void slab_records(const Params& p, unsigned char* sme
 
     // ---- (4)
     const int P = p.ncta;
-    const int RW = p.rec_words;
     for (int row = warp; row < mrows; row += nw) {
-        float* rec = p.part + ((size_t)row * P + cta) * RW;
+        auto rec = [&](int u) -> float2& { return *rec_pair(p.part, row, P, k, cta, u); };
         {
             const float s = warp_sum(lane < nw ? wsum_s[row * 16 + lane] : 0.f);      // fixed order: reproducible
-            if (lane == 0) *reinterpret_cast<float2*>(rec) = make_float2(cmax_s[row], s);
+            if (lane == 0) rec(0) = make_float2(cmax_s[row], s);
         }
         const int n = cnt_s[row];
         if (n <= kCand) {
-            // the (key, id) pairs go straight into the record: rank j to words 2 + 2 j, 3 + 2 j
+            // the (key, id) pairs go straight into the record
             const uint32_t* rk = ck + row * kCand;
             const int* ri = ci + row * kCand;
             for (int base = 0; base < n; base += 32) {
@@ -74,9 +119,9 @@ __device__ __forceinline__ void slab_records(const Params& p, unsigned char* sme
                 const int mi = i < n ? ri[i] : kNoId;
                 int rank = 0;
                 for (int j = 0; j < n; ++j) rank += better(rk[j], ri[j], mk, mi) ? 1 : 0;
-                if (i < n && rank < k) *reinterpret_cast<float2*>(rec + 2 + 2 * rank) = make_float2(__uint_as_float(mk), __int_as_float(mi));
+                if (i < n && rank < k) rec(1 + rank) = make_float2(__uint_as_float(mk), __int_as_float(mi));
             }
-            for (int j = n + lane; j < k; j += 32) *reinterpret_cast<float2*>(rec + 2 + 2 * j) = make_float2(__uint_as_float(0u), __int_as_float(kNoId));
+            for (int j = n + lane; j < k; j += 32) rec(1 + j) = make_float2(__uint_as_float(0u), __int_as_float(kNoId));
         } else {
             // Slow path (masses of equal logits, or logits in long ordered runs): k rounds over the
             // row, each taking the best logit that comes after the previous winner in the order;
@@ -95,49 +140,13 @@ __device__ __forceinline__ void slab_records(const Params& p, unsigned char* sme
                 const uint32_t wi = warp_min_u32(bk == wk ? (uint32_t)bi : 0xffffffffu);
                 lk = wk;
                 li = (int)wi;
-                if (lane == 0) *reinterpret_cast<float2*>(rec + 2 + 2 * j) = make_float2(__uint_as_float(wk), __int_as_float(wk != 0u ? (int)wi : kNoId));
+                if (lane == 0) rec(1 + j) = make_float2(__uint_as_float(wk), __int_as_float(wk != 0u ? (int)wi : kNoId));
                 if (wk == 0u) { lk = 0u; li = kNoId; }      // nothing left: later rounds stay empty
             }
         }
     }
 
-    // ---- arrival.  The CTAs take tickets from a counter that only counts up (the call's first ticket is
-    // p.ticket_base).  The last R of them to arrive merge: each takes every R-th row, waits until the counter
-    // shows that all P have arrived (they are already running: it is a wait of a microsecond, bounded all
-    // the same), and runs two tasks per row, a warp each: the row's log-sum-exp, and its k best entries.
-    if (!p.merge_inside) return;
-    __syncthreads();
-    if (tid == 0) *s_ticket = ticket_take(p.ticket) - p.ticket_base;
-    __syncthreads();
-    const int rows_at_once = max(1, nw >> 1);
-    const int R = min(P, (p.M + rows_at_once - 1) / rows_at_once);
-    const int me = (int)*s_ticket - (P - R);             // which of the R mergers this CTA is
-    if (me < 0) return;
-    if (me != R - 1) {
-        if (tid == 0) {
-            long long it = 0;
-            while (ld_acquire_gpu_u32(p.ticket) - p.ticket_base < (unsigned)P && ++it < kArrivalPolls) {}
-            if (it >= kArrivalPolls) atomicCAS(p.err, 0, ERR_WAIT_RECORD);
-        }
-        __syncthreads();
-    }
-    float* lse_s = reinterpret_cast<float*>(merge_area);                 // [16] by the CTA's own count of rows
-    uint32_t* ok_all = reinterpret_cast<uint32_t*>(lse_s + 16);          // [16 rows][32] ordered keys
-    int* oi_all = reinterpret_cast<int*>(ok_all + 16 * 32);              // [16 rows][32] their ids
-    uint32_t* mk = reinterpret_cast<uint32_t*>(oi_all + 16 * 32) + warp * 2 * kMergeCand;     // this warp's candidates
-    int* mi = reinterpret_cast<int*>(mk + kMergeCand);
-    const int mine = (p.M - me + R - 1) / R;             // rows me, me + R, ...
-    for (int task = warp; task < 2 * mine; task += nw) {
-        const int lr = task >> 1, row = me + lr * R;
-        if (P <= 5 * 32) merge_task<5>(p.part, P, RW, k, row, task & 1, lane, lse_s + lr, ok_all + lr * 32, oi_all + lr * 32, mk, mi, &cnt_s[warp]);
-        else merge_task<kMergeLists>(p.part, P, RW, k, row, task & 1, lane, lse_s + lr, ok_all + lr * 32, oi_all + lr * 32, mk, mi, &cnt_s[warp]);
-    }
-    __syncthreads();
-    for (int e = tid; e < mine * k; e += nt) {
-        const int lr = e / k, j = e - lr * k, row = me + lr * R;
-        p.ids[(size_t)row * k + j] = oi_all[lr * 32 + j];
-        p.logprobs[(size_t)row * k + j] = key2f(ok_all[lr * 32 + j]) - lse_s[lr];
-    }
+    if (p.merge_inside) merge_by_last_arrivals(p, s_ticket, merge_area);
 }
 
 // Epilogue of the head kernel.  The slab's logits lie in shared memory: logit (row, column c) is

@@ -10,8 +10,7 @@ namespace slimspec {
 typedef __nv_bfloat16 bf16;
 
 // One split-V partial record per (row, slab): running max, sum of exp(logit - max), and the
-// slab's k best (logit, id) pairs in (logit desc, id asc) order.
-// Layout in the context's scratch: float pm[P], ps[P], pv[P][k]; int pi[P][k] per row.
+// slab's k best (logit, id) pairs in (logit desc, id asc) order (layout: select.cuh).
 struct Scratch {
     float* z;            // fp32 code (or widened h): generic path [M][K]; one- and two-row streaming path: partial sums [splits][K][mt]
     uint32_t* zfrag;     // streaming path: the code, as fp32 or as tensor-core fragments (see stream.cu)
@@ -86,8 +85,15 @@ cudaError_t stream_head(const uint32_t* code, bool lowrank, const bf16* B, int M
                         int32_t* ids, float* logprobs, float* logits, const Scratch& s, int sm_count,
                         bool after_producer_kernel, int* launches, cudaStream_t st);
 
+// ---- streaming path, three to 64 rows, on the tcgen05 tensor cores (slab.cu) ----------------
+bool slab_ok(int M, bool lowrank, int K, int V, int k, int sm_count);
+cudaError_t slab_prepare();
+// logits = z W streamed once; z bf16 [M][K], z_lo (null: z is exact) its rounding remainder.
+cudaError_t slab_head(const bf16* z, const bf16* z_lo, const bf16* W, int M, int K, int V, int k, int mode, int32_t* ids, float* logprobs,
+                      float* logits, const Scratch& s, int sm_count, bool pdl, cudaStream_t st);
+
 // ---- the merge of split-V records as a kernel of its own (tensor path; streaming path with many rows)
-cudaError_t merge_records(const float* part, int M, int P, int RW, int k, int32_t* ids, float* logprobs, cudaStream_t st);
+cudaError_t merge_records(const float* part, int M, int P, int k, int32_t* ids, float* logprobs, cudaStream_t st);
 
 // ---- tensor-core path (larger M) ------------------------------------------------------
 // Shapes the tcgen05 kernels take: K a multiple of 64, N a multiple of 8 and >= 64, k <= 32 in top-k mode.

@@ -1,17 +1,27 @@
 // Selection of the k best (logit, id) pairs, shared by the streaming and the tensor-core path:
 // warp-level bounds, ordering by counting, and the merge of split-V records.
-// Records: per (row, slab) rec_words floats: maximum, sum of exp(logit - maximum), then k
-// (key, id) pairs in order, padded to a multiple of four words.
+// Records: 1 + k pairs of words per (row, slab): (maximum, sum of exp(logit - maximum)), then the slab's k
+// (key, id) pairs in order.  Pair u of all P slabs of a row lie next to each other: the merge, whose lanes take
+// a slab each, then reads whole lines.  (One record after the other it read a line per lane: eight rows took
+// 2.2 us to load, 5120 lines through one SM's L1, against 1.3 us; records of 32-byte sectors 1.7 us.)
 #pragma once
 #include "ptx.cuh"
 #include <float.h>
 
 namespace slimspec {
 
-static constexpr int kMergeCand = 128;                // candidates one row may park in the final merge
+static constexpr int kMaxK = 64;                      // largest k
+static constexpr int kMergeCand = 192;                // candidates one row may park in the final merge
 static constexpr int kMergeLists = 10;                // slab records a lane owns in the final merge
 static constexpr int kMaxRecords = 32 * kMergeLists;  // records per row the merge can take
 static constexpr int kNoId = 0x7fffffff;
+
+// where pair u of slab s of a row lies
+__host__ __device__ __forceinline__ size_t rec_row_pairs(int P, int k) { return (size_t)(1 + k) * P; }
+__device__ __forceinline__ float2* rec_pair(float* part, int row, int P, int k, int s, int u)
+{
+    return reinterpret_cast<float2*>(part) + (size_t)row * rec_row_pairs(P, k) + (size_t)u * P + s;
+}
 
 // ------------------------------------------------------------------------------------------
 // Selection.  Candidates are (key, id) with key = f2key(logit) and key 0 = none; the order is
@@ -31,20 +41,21 @@ __device__ __forceinline__ uint32_t warp_kth_largest(uint32_t key, int k, int la
     return __shfl_sync(0xffffffffu, key, __ffs(hit) - 1);
 }
 
-// The same for small k by k rounds of "take the maximum out": cheaper than counting up to about a dozen.
-__device__ __forceinline__ uint32_t warp_kth_largest_rounds(uint32_t key, int k, int lane)
+// A lower bound of the k-th largest of the warp's 32 lane values, by k rounds of "take the maximum out": exact unless
+// values are equal (equal ones leave together, which only lowers the bound); 0 if there are fewer than k distinct ones.
+// Cheaper than counting up to about a dozen.
+__device__ __forceinline__ uint32_t warp_kth_rounds(uint32_t key, int k)
 {
     uint32_t kth = 0u;
     for (int j = 0; j < k; ++j) {
         kth = warp_max_u32(key);
-        const unsigned eq = __ballot_sync(0xffffffffu, key == kth);
-        if (lane == __ffs(eq) - 1) key = 0u;
+        key = key == kth ? 0u : key;
     }
     return kth;
 }
 __device__ __forceinline__ uint32_t warp_kth_largest_any(uint32_t key, int k, int lane)
 {
-    return k <= 12 ? warp_kth_largest_rounds(key, k, lane) : warp_kth_largest(key, k, lane);
+    return k <= 12 ? warp_kth_rounds(key, k) : warp_kth_largest(key, k, lane);
 }
 
 // The same over 64 values, two per lane (value a has index lane, value b index lane + 32).
@@ -67,25 +78,78 @@ __device__ __forceinline__ uint32_t warp_kth_largest64(uint32_t a, uint32_t b, i
     return hit_a ? va : vb;
 }
 
-// n candidates in shared memory, in any order, distinct ids.  The warp writes the min(n, k)
-// best in order to (ok, oi) and pads up to k with empty entries.  By counting: a candidate's
-// place is the number of candidates ahead of it.
-__device__ __forceinline__ void warp_rank_select(const uint32_t* ck, const int* ci, int n, int k, uint32_t* ok,
-                                                 int* oi, int lane)
+// A lower bound of the k-th largest (k <= 32 NV) of 32 NV keys, NV per lane, less than 32 NV units of the key below
+// it (the low bits of a key give way to its place, so that the words are distinct and a rank is a plain
+// count).  The words are passed round through s (32 NV of them, of this warp, 16-byte aligned): broadcast
+// reads of four words at a time, where shuffles took four times as long.
+template <int NV>
+__device__ __forceinline__ uint32_t warp_kth_bound(const uint32_t (&key)[NV], int k, int lane, uint32_t* s)
 {
+    constexpr uint32_t LOW = NV == 1 ? 31u : NV == 2 ? 63u : NV <= 4 ? 127u : NV <= 8 ? 255u : 511u;
+    uint32_t u[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) {
+        u[v] = (key[v] & ~LOW) | (LOW - (uint32_t)(lane + 32 * v));
+        s[lane + 32 * v] = u[v];
+    }
+    __syncwarp();
+    int rank[NV];
+#pragma unroll
+    for (int v = 0; v < NV; ++v) rank[v] = 0;
+#pragma unroll 8
+    for (int i = 0; i < 8 * NV; ++i) {
+        const uint4 o = reinterpret_cast<const uint4*>(s)[i];
+#pragma unroll
+        for (int v = 0; v < NV; ++v) rank[v] += (o.x > u[v]) + (o.y > u[v]) + (o.z > u[v]) + (o.w > u[v]);
+    }
+    uint32_t mine = 0u;          // exactly one of the words has rank k - 1
+#pragma unroll
+    for (int v = 0; v < NV; ++v) mine = rank[v] == k - 1 ? u[v] : mine;
+    const uint32_t r = __reduce_max_sync(0xffffffffu, mine) & ~LOW;
+    __syncwarp();
+    return r;
+}
+
+// A candidate as one word: larger is better (key descending, id ascending).  0: none.
+__device__ __forceinline__ unsigned long long cand_word(uint32_t key, int id)
+{
+    return ((unsigned long long)key << 32) | (uint32_t)~(uint32_t)id;
+}
+__device__ __forceinline__ uint32_t cand_key(unsigned long long c) { return (uint32_t)(c >> 32); }
+__device__ __forceinline__ int cand_id(unsigned long long c) { return (int)~(uint32_t)c; }
+
+// Sum of the values of the lanes before this one, and of all lanes.
+__device__ __forceinline__ int warp_exclusive_sum(int v, int lane, int* total)
+{
+    int x = v;
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {
+        const int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+    }
+    *total = __shfl_sync(0xffffffffu, x, 31);
+    return x - v;
+}
+
+// n distinct candidate words in shared memory (16-byte aligned, room for n + 3 words), in any order: the warp hands
+// the min(n, k) best to put(rank, word), by counting: a candidate's rank is the number of better ones.
+template <class Put>
+__device__ __forceinline__ void warp_rank_words(unsigned long long* c, int n, int k, int lane, Put put)
+{
+    if (lane < 3) c[n + lane] = 0ull;          // the reads below go four at a time
+    __syncwarp();
     for (int base = 0; base < n; base += 32) {
         const int i = base + lane;
-        const uint32_t mk = i < n ? ck[i] : 0u;
-        const int mi = i < n ? ci[i] : kNoId;
+        const unsigned long long mine = i < n ? c[i] : ~0ull;
         int rank = 0;
-        for (int j = 0; j < n; ++j) {
-            const uint32_t kj = ck[j];
-            const int ij = ci[j];
-            rank += (kj > mk || (kj == mk && ij < mi)) ? 1 : 0;
+        for (int j = 0; j < n; j += 4) {
+            const ulonglong2 a = *reinterpret_cast<const ulonglong2*>(c + j);
+            const ulonglong2 b = *reinterpret_cast<const ulonglong2*>(c + j + 2);
+            rank += (a.x > mine) + (a.y > mine) + (b.x > mine) + (b.y > mine);
         }
-        if (i < n && rank < k) { ok[rank] = mk; oi[rank] = mi; }
+        if (i < n && rank < k) put(rank, mine);
     }
-    for (int j = n + lane; j < k; j += 32) { ok[j] = 0u; oi[j] = kNoId; }
+    __syncwarp();
 }
 
 // is (ka, ia) strictly after (kb, ib) in the order, i.e. a worse candidate?
@@ -100,21 +164,22 @@ __device__ __forceinline__ bool better(uint32_t ka, int ia, uint32_t kb, int ib)
 }
 
 // ------------------------------------------------------------------------------------------
-// ------------------------------------------------------------------------------------------
 // One task of the merge, run by one warp: kind 0 = the row's log-sum-exp from the records'
-// (maximum, sum-exp) pairs, written to *lse_out; kind 1 = its k best entries.  A lane owns the records lane,
-// lane + 32, ... (NL of them at most) and keeps what it loads in registers: one round trip to the L2.
+// (maximum, sum-exp) pairs, written to *lse_out; kind 1 = its k best entries, in order, to out, padded
+// with empty ones (key 0).  A lane owns the records lane, lane + 32, ... (NL of them at most) and keeps what it loads
+// in registers: one round trip to the L2.  area: kMergeWarpBytes of shared memory of this warp, 16-byte aligned.
+static constexpr int kMergeWarpBytes = kMaxRecords * 4 + (kMergeCand + 4) * 8 + 16;
 template <int NL>
-__device__ __forceinline__ void merge_task(const float* part, int P, int RW, int k, int row, int kind, int lane, float* lse_out,
-                                           uint32_t* ok, int* oi, uint32_t* mk, int* mi, int* cnt)
+__device__ __forceinline__ void merge_task(const float* part, int P, int k, int row, int kind, int lane, float* lse_out,
+                                           unsigned long long* out, unsigned char* area)
 {
-    const float* rows = part + (size_t)row * P * RW;
+    const float2* rows = reinterpret_cast<const float2*>(part) + (size_t)row * rec_row_pairs(P, k);
     if (kind == 0) {
         float2 ms[NL];
 #pragma unroll
         for (int q = 0; q < NL; ++q) {
             const int s = lane + 32 * q;
-            ms[q] = s < P ? __ldcg(reinterpret_cast<const float2*>(rows + (size_t)s * RW)) : make_float2(-FLT_MAX, 0.f);
+            ms[q] = s < P ? __ldcg(rows + s) : make_float2(-FLT_MAX, 0.f);
         }
         float gm = -FLT_MAX;
 #pragma unroll
@@ -127,56 +192,72 @@ __device__ __forceinline__ void merge_task(const float* part, int P, int RW, int
         if (lane == 0) *lse_out = gm + __logf(gs);
         return;
     }
-    // the first three entries of every record (words 2..7), then the bound: at least k entries
-    // reach the k-th largest of the lanes' best first entries
-    float2 e0[NL];
-    float4 e12[NL];
+    uint32_t* s32 = reinterpret_cast<uint32_t*>(area);
+    unsigned long long* cand = reinterpret_cast<unsigned long long*>(s32 + kMaxRecords);
+    int* cnt = reinterpret_cast<int*>(cand + kMergeCand + 4);
+    // the first three entries of every record, then the bound
+    const float2 none = make_float2(0.f, __int_as_float(kNoId));
+    float2 e0[NL], e1[NL], e2[NL];
 #pragma unroll
     for (int q = 0; q < NL; ++q) {
         const int s = lane + 32 * q;
-        e0[q] = make_float2(0.f, __int_as_float(kNoId));
-        e12[q] = make_float4(0.f, __int_as_float(kNoId), 0.f, __int_as_float(kNoId));
-        if (s < P) {
-            e0[q] = __ldcg(reinterpret_cast<const float2*>(rows + (size_t)s * RW + 2));
-            if (k >= 2) e12[q] = __ldcg(reinterpret_cast<const float4*>(rows + (size_t)s * RW + 4));
-        }
+        e0[q] = s < P ? __ldcg(rows + P + s) : none;
+        e1[q] = s < P && k >= 2 ? __ldcg(rows + 2 * P + s) : none;
+        e2[q] = s < P && k >= 3 ? __ldcg(rows + 3 * P + s) : none;
     }
-    uint32_t hk = 0u;
+    // Up to k = 24 the k-th largest of the lanes' best entries: with 24 of 32 lanes about 44 entries reach it.
+    // Beyond, every record's best entry counts by itself (k = 64 of 148 records: about 84 entries).
+    uint32_t kth;
+    if (k <= 24) {
+        uint32_t hk[1] = {0u};
 #pragma unroll
-    for (int q = 0; q < NL; ++q) hk = max(hk, __float_as_uint(e0[q].x));
-    const uint32_t kth = warp_kth_largest_any(hk, min(k, 32), lane);
-    if (lane == 0) *cnt = 0;
-    __syncwarp();
+        for (int q = 0; q < NL; ++q) hk[0] = max(hk[0], __float_as_uint(e0[q].x));
+        kth = k <= 12 ? warp_kth_rounds(hk[0], k) : warp_kth_bound<1>(hk, k, lane, s32);
+    } else {
+        uint32_t hk[NL];
 #pragma unroll
-    for (int q = 0; q < NL; ++q) {
-        const uint32_t k0 = __float_as_uint(e0[q].x);
-        if (k0 != 0u && k0 >= kth) {
-            int pos = atomicAdd(cnt, 1);
-            if (pos < kMergeCand) { mk[pos] = k0; mi[pos] = __float_as_int(e0[q].y); }
-            const uint32_t k1 = __float_as_uint(e12[q].x);
-            if (k >= 2 && k1 != 0u && k1 >= kth) {          // the record's list is in order: rarely more than one entry
-                pos = atomicAdd(cnt, 1);
-                if (pos < kMergeCand) { mk[pos] = k1; mi[pos] = __float_as_int(e12[q].y); }
-                const uint32_t k2 = __float_as_uint(e12[q].z);
-                if (k >= 3 && k2 != 0u && k2 >= kth) {
-                    pos = atomicAdd(cnt, 1);
-                    if (pos < kMergeCand) { mk[pos] = k2; mi[pos] = __float_as_int(e12[q].w); }
-                    const float* rec = rows + (size_t)(lane + 32 * q) * RW;
-                    for (int j = 3; j < k; ++j) {
-                        const float2 en = __ldcg(reinterpret_cast<const float2*>(rec + 2 + 2 * j));
-                        const uint32_t kj = __float_as_uint(en.x);
-                        if (kj == 0u || kj < kth) break;
-                        pos = atomicAdd(cnt, 1);
-                        if (pos < kMergeCand) { mk[pos] = kj; mi[pos] = __float_as_int(en.y); }
-                    }
+        for (int q = 0; q < NL; ++q) hk[q] = __float_as_uint(e0[q].x);
+        kth = warp_kth_bound<NL>(hk, k, lane, s32);
+    }
+    kth = max(kth, 1u);                      // empty entries (key 0) never count
+    // the entries that reach the bound, by ballot: the first ones, then, where any do, the second and third ones (a record's
+    // list is in order, so its later entries matter only where the earlier ones reach the bound)
+    const unsigned below = (1u << lane) - 1u;
+    int n = 0;
+    bool second = false, third = false;
+    auto park = [&](float2 e) {
+        const bool in = __float_as_uint(e.x) >= kth;
+        const unsigned b = __ballot_sync(0xffffffffu, in);
+        const int pos = n + __popc(b & below);
+        if (in && pos < kMergeCand) cand[pos] = cand_word(__float_as_uint(e.x), __float_as_int(e.y));
+        n += __popc(b);
+    };
+#pragma unroll
+    for (int q = 0; q < NL; ++q) { park(e0[q]); second = second || __float_as_uint(e1[q].x) >= kth; }
+    if (__any_sync(0xffffffffu, second)) {
+#pragma unroll
+        for (int q = 0; q < NL; ++q) { park(e1[q]); third = third || __float_as_uint(e2[q].x) >= kth; }
+        if (__any_sync(0xffffffffu, third)) {
+            if (lane == 0) *cnt = n;
+            __syncwarp();
+#pragma unroll 1
+            for (int s = lane; s < P; s += 32) {
+                for (int j = 2; j < k; ++j) {
+                    const float2 en = __ldcg(rows + (size_t)(1 + j) * P + s);
+                    const uint32_t kj = __float_as_uint(en.x);
+                    if (kj < kth) break;
+                    const int at = atomicAdd(cnt, 1);
+                    if (at < kMergeCand) cand[at] = cand_word(kj, __float_as_int(en.y));
                 }
             }
+            __syncwarp();
+            n = *cnt;
         }
     }
     __syncwarp();
-    const int n = *cnt;
     if (n <= kMergeCand) {
-        warp_rank_select(mk, mi, n, k, ok, oi, lane);
+        warp_rank_words(cand, n, k, lane, [&](int rank, unsigned long long c) { out[rank] = c; });
+        for (int j = n + lane; j < k; j += 32) out[j] = cand_word(0u, kNoId);
     } else {
         // slow path: k rounds over every entry of the row's records, each round taking the best
         // entry after the previous winner
@@ -186,19 +267,19 @@ __device__ __forceinline__ void merge_task(const float* part, int P, int RW, int
             uint32_t bk = 0u;
             int bi = kNoId;
             for (int s = lane; s < P; s += 32) {
-                const float* rec = rows + (size_t)s * RW;
                 for (int e = 0; e < k; ++e) {
-                    const float2 en = __ldcg(reinterpret_cast<const float2*>(rec + 2 + 2 * e));
+                    const float2 en = __ldcg(rows + (size_t)(1 + e) * P + s);
                     const uint32_t ke = __float_as_uint(en.x);
                     const int ie = __float_as_int(en.y);
-                    if (ke != 0u && after(ke, ie, lk, li) && better(ke, ie, bk, bi)) { bk = ke; bi = ie; }
+                    if (ke == 0u || !better(ke, ie, bk, bi)) break;        // the list is in order: nothing better follows ...
+                    if (after(ke, ie, lk, li)) { bk = ke; bi = ie; break; }  // ... and the first one after the winner is its best
                 }
             }
             const uint32_t wk = warp_max_u32(bk);
             const uint32_t wi = warp_min_u32(bk == wk ? (uint32_t)bi : 0xffffffffu);
             lk = wk;
             li = (int)wi;
-            if (lane == 0) { ok[j] = wk; oi[j] = wk != 0u ? (int)wi : kNoId; }
+            if (lane == 0) out[j] = cand_word(wk, wk != 0u ? (int)wi : kNoId);
             if (wk == 0u) { lk = 0u; li = kNoId; }
         }
     }

@@ -44,11 +44,10 @@ struct HeadParams {
     int nkb;                  // 16-row blocks of the matrix: ceil(K / 16)
     int kb_chunk, nchunks;    // blocks of code fragments per shared-memory chunk, chunks
     unsigned int zarea_bytes; // shared memory the code takes
-    int rec_words;            // words per record: max, sum-exp, k (key, id) pairs, padded to 4
     int32_t* ids;
     float* logprobs;
     float* logits;
-    float* part;              // records [M][ncta * npass][rec_words]
+    float* part;              // records (see select.cuh)
     unsigned int* ticket;
     unsigned int ticket_base; // what the counter read when the call began
     int* err;
@@ -476,21 +475,20 @@ __global__ void __launch_bounds__(256, 2) k_stream_head_mma(const HeadParams p) 
 
 // ------------------------------------------------------------------------------------------
 struct Geometry {
-    int ncta, units_base, units_rem, rec_words;
+    int ncta, units_base, units_rem;
     int nch, pitch_units, ns, nkb, kb_chunk, nchunks, warps;
     size_t zarea_bytes, smem;
 };
 
 static constexpr size_t kHeadSmemMax = 226 * 1024;
 
-static size_t merge_bytes(int) { return (size_t)(16 + 2 * 16 * 32 + 16 * 2 * kMergeCand) * 4; }
+static size_t merge_bytes(int) { return merge_area_bytes(16, 8); }
 
 // zparts: 1 or 2 parts of code fragments (tensor-core kernel)
 static bool geometry(int M, int zparts, int K, int V, int k, int sm_count, Geometry* g)
 {
     if (V % 8 != 0 || K < 1 || k > 32 || k < 1 || M < 1 || M > 16) return false;
     const int units = V / 8;
-    g->rec_words = (2 + 2 * k + 3) / 4 * 4;
     const size_t fixed0 = ((kEpFixedBytes + 127) / 128) * 128;
     const int mt = M <= 8 ? 8 : 16;
     // two CTAs per SM
@@ -711,7 +709,6 @@ cudaError_t stream_head(const uint32_t* zfrag, bool lowrank, const bf16* B, int 
     memset(&hp, 0, sizeof(hp));
     hp.zfrag = zfrag; hp.B = B; hp.M = M; hp.K = K; hp.V = V; hp.k = k; hp.mode = mode;
     hp.ncta = g.ncta; hp.units_base = g.units_base; hp.units_rem = g.units_rem;
-    hp.rec_words = g.rec_words;
     hp.zarea_bytes = (unsigned int)g.zarea_bytes;
     hp.ids = ids; hp.logprobs = logprobs; hp.logits = logits;
     hp.part = s.part; hp.ticket = s.tickets; hp.err = s.err;

@@ -25,7 +25,6 @@ static constexpr int kFmaMaxColThreads = 256;   // threads across a slab's colum
 static constexpr int kFmaMaxCtas = 256;         // most slabs
 static constexpr int kFmaZChunkBytes = 64 * 1024;   // shared memory for the code, as (z, z) pairs
 static constexpr int kFmaEpFixed = (kEpFixedBytes + 127) / 128 * 128;      // the epilogue's fixed area
-static constexpr int kFmaMergeBytes = (16 + 2 * 16 * 32 + 8 * 2 * kMergeCand) * 4 + 64;   // the last CTA's merge: up to eight tasks
 #ifndef SLIMSPEC_FMA4_MIN_A
 #define SLIMSPEC_FMA4_MIN_A (4u << 20)
 #endif
@@ -48,7 +47,6 @@ struct FmaParams {
     int units_base, units_rem;   // V/8 column units: slab c has units_base + (c < units_rem)
     int ct, rg;           // column threads (multiple of 32) and row groups: blockDim = ct * rg
     int kc;               // rows of the code per shared-memory chunk (K, or a multiple of rg * U)
-    int rec_words;        // words per split-V record: max, sum-exp, k (key, id) pairs, padded to 4
     int merge_inside;     // 1: the last CTA to arrive merges the records
     // the down-projection, shared out among the CTAs as jobs: job j = (split j / code_units, unit j % code_units)
     int njobs;
@@ -60,7 +58,7 @@ struct FmaParams {
     int32_t* ids;
     float* logprobs;
     float* logits;
-    float* part;          // split-V records [M][ncta][rec_words]
+    float* part;          // split-V records (see select.cuh)
     unsigned int* ticket;
     unsigned int ticket_base;   // what the counter read when the call began
     int* err;
@@ -353,7 +351,7 @@ __global__ void __launch_bounds__(512, 1) k_fma_head(const FmaParams p)
 static int fma_pick_mt(int M) { return M <= 2 ? M : 4; }
 
 struct FmaGeometry {
-    int ncta, units_base, units_rem, max_units, ct, rg, u, kc, rec_words, threads;
+    int ncta, units_base, units_rem, max_units, ct, rg, u, kc, threads;
     int njobs, code_units, nsplit, job_rows, red_bytes;
     size_t smem;
 };
@@ -386,8 +384,9 @@ static bool fma_geometry(int mt, int d, int r, int V, int k, int sm_count, FmaGe
         g->kc = kc_max / (g->rg * g->u) * (g->rg * g->u);
         if (g->kc < 1) return false;
     }
-    g->rec_words = (2 + 2 * k + 3) / 4 * 4;
-    g->red_bytes = g->threads * mt * 32 > kFmaMergeBytes ? g->threads * mt * 32 : kFmaMergeBytes;
+    g->red_bytes = g->threads * mt * 32;
+    const int merge = (merge_area_bytes(mt, 2 * mt) + 127) / 128 * 128;      // the last CTA's merge: two tasks a row
+    if (g->red_bytes < merge) g->red_bytes = merge;
     g->smem = (size_t)kFmaEpFixed + (size_t)mt * kCand * 8 + g->red_bytes + (size_t)g->kc * mt * 8;
     if (g->smem > 200 * 1024) return false;
     // the down-projection's jobs: one 16-byte unit of A's columns each; the rows of A are split while
@@ -448,7 +447,7 @@ cudaError_t fma_head(const bf16* h, const bf16* A, const bf16* B, int M, int mt,
     FmaParams hp;
     hp.h = h; hp.A = A; hp.B = B; hp.M = M; hp.d = d; hp.K = K; hp.V = V; hp.k = k; hp.mode = mode;
     hp.ncta = g.ncta; hp.units_base = g.units_base; hp.units_rem = g.units_rem;
-    hp.ct = g.ct; hp.rg = g.rg; hp.kc = g.kc; hp.rec_words = g.rec_words; hp.merge_inside = 1;
+    hp.ct = g.ct; hp.rg = g.rg; hp.kc = g.kc; hp.merge_inside = 1;
     hp.njobs = g.njobs; hp.code_units = g.code_units; hp.nsplit = g.nsplit; hp.job_rows = g.job_rows;
     hp.zpart = s.zq; hp.epoch = epoch; hp.red_bytes = g.red_bytes;
     hp.ids = ids; hp.logprobs = logprobs; hp.logits = logits;

@@ -12,7 +12,7 @@
 #include "kernels.h"
 #include "ptx.cuh"
 #include "select.cuh"
-#include <cuda.h>
+#include "tmap.h"
 #include <float.h>
 #include <string.h>
 
@@ -50,7 +50,6 @@ struct alignas(64) TcParams {
     uint32_t* smax;         // mode 3 output
     const uint32_t* thr0;   // mode 0: per-row lower bound (key - 1) of the k-th largest logit, or null
     int k;
-    int rec_words;
     int ns;                 // stages of the W ring
     int nsx;                // stages of the X ring (unused when X is resident)
     int xbox_bytes;         // bytes of one X box: (rows of the box, 8..128) x 128; rows past the box are garbage in,
@@ -58,7 +57,7 @@ struct alignas(64) TcParams {
     int split;              // 1: X = X_hi + X_lo (two bf16 matrices): two MMAs per step into one accumulator
     int xres;               // 1: the row block's whole X (K <= 512) is loaded once and stays in shared memory
     float* out;
-    float* part;            // records [M][2 * gct][rec_words]: two column halves per CTA
+    float* part;            // records of 2 gct slabs a row (see select.cuh): two column halves per CTA
     int* err;
 };
 
@@ -394,12 +393,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
                 si[j] = ci[j];
             }
             topk_compact(sv, si, cnt, k, thr);
-            float* rec = p.part + ((size_t)m * (2 * p.gct) + 2 * cg + half) * p.rec_words;
-            rec[0] = run_max;
-            rec[1] = run_sum;
+            const int P = 2 * p.gct;
+            *rec_pair(p.part, m, P, k, 2 * cg + half, 0) = make_float2(run_max, run_sum);
             for (int j = 0; j < k; ++j)      // (key, id) pairs; -0 and +0 rank alike
-                *reinterpret_cast<float2*>(rec + 2 + 2 * j) =
-                    make_float2(__uint_as_float(j < cnt ? f2key(sv[j] + 0.f) : 0u), __int_as_float(j < cnt ? si[j] : kTcNoId));
+                *rec_pair(p.part, m, P, k, 2 * cg + half, 1 + j) = make_float2(__uint_as_float(j < cnt ? f2key(sv[j] + 0.f) : 0u), __int_as_float(j < cnt ? si[j] : kTcNoId));
         }
     }
     // ---- teardown: every role is past its last use of tensor memory
@@ -460,62 +457,28 @@ __global__ void __launch_bounds__(256) k_tc_thr0(const uint32_t* __restrict__ sm
 // Merge the P per-slab records of each row.  Two rows per CTA, two warps per row: one takes the
 // row's log-sum-exp, the other its k best entries (bound from the records' first entries, the few
 // entries above it ordered by counting).
-__global__ void __launch_bounds__(128) k_tc_merge(const float* __restrict__ part, int M, int P, int RW, int k,
+__global__ void __launch_bounds__(128) k_tc_merge(const float* __restrict__ part, int M, int P, int k,
                                                   int32_t* __restrict__ ids, float* __restrict__ logprobs)
 {
     __shared__ float lse_s[2];
-    __shared__ uint32_t ok_s[2][32];
-    __shared__ int oi_s[2][32];
-    __shared__ uint32_t mk_s[4][kMergeCand];
-    __shared__ int mi_s[4][kMergeCand];
-    __shared__ int cnt_s[4];
+    __shared__ unsigned long long out_s[2][kMaxK];
+    __shared__ __align__(16) unsigned char area_s[4][kMergeWarpBytes];
     pdl_launch_dependents();     // the first kernel of the next call may come up behind this one
     pdl_wait();
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
     const int r2 = warp >> 1, row = blockIdx.x * 2 + r2;
     if (row < M) {
-        if (P <= 5 * 32) merge_task<5>(part, P, RW, k, row, warp & 1, lane, &lse_s[r2], ok_s[r2], oi_s[r2], mk_s[warp], mi_s[warp], &cnt_s[warp]);
-        else merge_task<kMergeLists>(part, P, RW, k, row, warp & 1, lane, &lse_s[r2], ok_s[r2], oi_s[r2], mk_s[warp], mi_s[warp], &cnt_s[warp]);
+        if (P <= 5 * 32) merge_task<5>(part, P, k, row, warp & 1, lane, &lse_s[r2], out_s[r2], area_s[warp]);
+        else merge_task<kMergeLists>(part, P, k, row, warp & 1, lane, &lse_s[r2], out_s[r2], area_s[warp]);
     }
     __syncthreads();
     if ((warp & 1) == 0 && row < M && lane < k) {
-        ids[(size_t)row * k + lane] = oi_s[r2][lane];
-        logprobs[(size_t)row * k + lane] = key2f(ok_s[r2][lane]) - lse_s[r2];
+        ids[(size_t)row * k + lane] = cand_id(out_s[r2][lane]);
+        logprobs[(size_t)row * k + lane] = key2f(cand_key(out_s[r2][lane])) - lse_s[r2];
     }
 }
 
 // ------------------------------------------------------------------------------------------
-typedef CUresult (*EncodeTiledFn)(CUtensorMap*, CUtensorMapDataType, cuuint32_t, void*, const cuuint64_t*,
-                                  const cuuint64_t*, const cuuint32_t*, const cuuint32_t*, CUtensorMapInterleave,
-                                  CUtensorMapSwizzle, CUtensorMapL2promotion, CUtensorMapFloatOOBfill);
-
-static EncodeTiledFn encode_fn()
-{
-    static EncodeTiledFn fn = nullptr;
-    if (!fn) {
-        void* ptr = nullptr;
-        cudaDriverEntryPointQueryResult qr;
-        if (cudaGetDriverEntryPoint("cuTensorMapEncodeTiled", &ptr, cudaEnableDefault, &qr) == cudaSuccess &&
-            qr == cudaDriverEntryPointSuccess)
-            fn = (EncodeTiledFn)ptr;
-    }
-    return fn;
-}
-
-// bf16 matrix [rows][cols] (cols contiguous), box = box_cols x box_rows, 128-byte swizzle, zero fill
-static bool make_map(CUtensorMap* map, const void* base, int rows, int cols, int box_cols, int box_rows)
-{
-    EncodeTiledFn fn = encode_fn();
-    if (!fn) return false;
-    cuuint64_t dims[2] = {(cuuint64_t)cols, (cuuint64_t)rows};
-    cuuint64_t strides[1] = {(cuuint64_t)cols * 2};
-    cuuint32_t box[2] = {(cuuint32_t)box_cols, (cuuint32_t)box_rows};
-    cuuint32_t es[2] = {1, 1};
-    return fn(map, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 2, const_cast<void*>(base), dims, strides, box, es,
-              CU_TENSOR_MAP_INTERLEAVE_NONE, CU_TENSOR_MAP_SWIZZLE_128B, CU_TENSOR_MAP_L2_PROMOTION_L2_256B,
-              CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE) == CUDA_SUCCESS;
-}
-
 bool tensor_ok(int M, int K, int N, int k, int mode)
 {
     if (M < 1 || K < kTcKChunk || K % kTcKChunk != 0 || N % 8 != 0 || N < 64) return false;
@@ -525,29 +488,10 @@ bool tensor_ok(int M, int K, int N, int k, int mode)
 
 static constexpr size_t kTcSmemMax = 227 * 1024 - 512;   // dynamic shared memory per CTA (a little static on top)
 
-// Launch with (or without) the programmatic-dependent-launch attribute: the kernel may start while
-// the one before it in the stream is still running and meets it at griddepcontrol.wait.
-template <typename... KArgs, typename... Args>
-static cudaError_t launch_chain(void (*kern)(KArgs...), int grid, int block, size_t smem, bool pdl, cudaStream_t st,
-                                Args... args)
-{
-    cudaLaunchConfig_t cfg = {};
-    cfg.gridDim = dim3(grid);
-    cfg.blockDim = dim3(block);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kern, args...);
-}
-
 // Merge kernel: P split-V records per row -> ids / log-probs; launched early behind the kernel that writes them.
-cudaError_t merge_records(const float* part, int M, int P, int RW, int k, int32_t* ids, float* logprobs, cudaStream_t st)
+cudaError_t merge_records(const float* part, int M, int P, int k, int32_t* ids, float* logprobs, cudaStream_t st)
 {
-    return launch_chain(k_tc_merge, (M + 1) / 2, 128, 0, true, st, part, M, P, RW, k, ids, logprobs);
+    return launch_chain(k_tc_merge, (M + 1) / 2, 128, 0, true, st, part, M, P, k, ids, logprobs);
 }
 
 // Chooses the ring depth (and whether X can stay resident) and launches.
@@ -582,7 +526,7 @@ bool tensor_records_fit(int M, int N, int k, const Scratch& s, int sm_count)
     if (gct < 1) gct = 1;
     if (gct > nct) gct = nct;
     if (gct > kMaxRecords / 2) gct = kMaxRecords / 2;
-    return (size_t)M * 2 * gct * ((2 + 2 * k + 3) / 4 * 4) <= s.part_elems;
+    return (size_t)M * 2 * rec_row_pairs(2 * gct, k) <= s.part_elems;
 }
 
 // out = X W through the tensor cores.  mode 0: top-k records then merge into ids / logprobs;
@@ -617,11 +561,10 @@ cudaError_t tensor_head(const bf16* X, const bf16* Xlo, const bf16* W, int M, in
     if (p.gct > kMaxRecords / 2) p.gct = kMaxRecords / 2;       // the merge takes up to 320 lists per row
     p.mode = mode;
     p.k = k;
-    p.rec_words = (2 + 2 * k + 3) / 4 * 4;
     p.out = logits;
     p.part = s.part;
     p.err = s.err;
-    if (mode == 0 && (size_t)M * 2 * p.gct * p.rec_words > s.part_elems) return cudaErrorInvalidValue;
+    if (mode == 0 && (size_t)M * 2 * rec_row_pairs(2 * p.gct, k) > s.part_elems) return cudaErrorInvalidValue;
     cudaError_t e;
     if (mode == 0) {
         // A bound below each row's k-th largest logit, from the first sample tiles of the vocabulary:
@@ -656,7 +599,7 @@ cudaError_t tensor_head(const bf16* X, const bf16* Xlo, const bf16* W, int M, in
     if (ev1 && (e = cudaEventRecord(ev1, st)) != cudaSuccess) return e;
     *launches += 1;
     if (mode == 0) {
-        e = merge_records(s.part, M, 2 * p.gct, p.rec_words, k, ids, logprobs, st);
+        e = merge_records(s.part, M, 2 * p.gct, k, ids, logprobs, st);
         *launches += 1;
     }
     return e;
