@@ -31,9 +31,10 @@
  *     launch and start reading weights while the kernel before the call may still be
  *     running; a kernel that rewrites weights directly before a call (a dequantisation, a
  *     weight swap) must be followed by an event or stream synchronisation.
- *   - The generic path (shapes the fast kernels do not take, or forced) keeps an M x V fp32
- *     buffer in the context for its top-k call and grows it on demand: such a call may
- *     allocate and synchronise the device.  The fast paths never do.
+ *   - The generic path, forced (or for the few shapes that nothing else takes: more than about
+ *     170000 columns in an odd layout), keeps an M x V fp32 buffer in the context for its top-k
+ *     call and grows it on demand: such a call may allocate and synchronise the device.  No other
+ *     call does.
  *   - Return value: SLIMSPEC_OK or a negative status; nothing is launched on an argument
  *     error.  There is no CPU fallback: every step runs in CUDA kernels.
  *   - 1 <= k <= min(V, SLIMSPEC_MAX_K).  Inputs holding NaN or infinity give unspecified
@@ -62,7 +63,8 @@ extern "C" {
 
 /* execution paths (slimspec_force_path) */
 #define SLIMSPEC_PATH_AUTO 0        /* chosen per (M, shapes) from measured timings            */
-#define SLIMSPEC_PATH_GENERIC 1     /* any shape; one thread per logit; slow                   */
+#define SLIMSPEC_PATH_GENERIC 1     /* any shape.  Forced: one thread per logit, slow.  Chosen by AUTO:
+                                       the streaming tensor-core kernel, up to 64 rows a launch */
 #define SLIMSPEC_PATH_STREAM 2      /* split-V weight-streaming kernels (M <= 16 per launch)   */
 #define SLIMSPEC_PATH_TENSOR 3      /* tcgen05 / TMEM tensor-core kernels (large M)            */
 

@@ -94,8 +94,9 @@ extern "C" int slimspec_create(slimspec_ctx** out, int max_M, int max_d, int max
     ok = ok && cudaMalloc(&c->s.zfrag, stream_code_bytes(max_d)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->s.zq, fma_code_words(max_d) * sizeof(uint2)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->s.zpart, zpart_elems * sizeof(float)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->s.zb, 2 * mpad128 * (size_t)max_d * sizeof(bf16)) == cudaSuccess;
-    if (ok) c->s.zb_lo = c->s.zb + mpad128 * (size_t)max_d;
+    const size_t dpad = (size_t)round_up(max_d, 8);          // rows on a pitch that TMA takes
+    ok = ok && cudaMalloc(&c->s.zb, (2 * mpad128 + kSlabRows) * dpad * sizeof(bf16)) == cudaSuccess;
+    if (ok) { c->s.zb_lo = c->s.zb + mpad128 * dpad; c->s.zb_lo2 = c->s.zb_lo + mpad128 * dpad; }
     ok = ok && cudaMalloc(&c->s.smax, 64 * mpad128 * sizeof(uint32_t)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->s.thr0, mpad128 * sizeof(uint32_t)) == cudaSuccess;
     c->s.smax_elems = 64 * mpad128;
@@ -272,6 +273,41 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
     if (path == SLIMSPEC_PATH_STREAM && !stream_ok) return SLIMSPEC_ERR_ALIGN;
     c->last_path = path;
 
+    // The shapes that no fast path takes (an odd vocabulary, k > 32, unaligned pointers): chosen automatically they run on the
+    // slab kernel too, its weights fed through registers where TMA does not take them, the code in three parts
+    // (all of fp32, as before), 64 rows a launch.  Forced, they run on the plain kernels, a second implementation.
+    // (5 rows, d = 2880, r = 360, V = 50257: 950 us on the plain kernels, 31.9 us here.)
+    int any_rows = 0;
+    if (path == SLIMSPEC_PATH_GENERIC && c->forced_path == SLIMSPEC_PATH_AUTO && ((uintptr_t)h & 1) == 0 && ((uintptr_t)Bm & 1) == 0) {
+        any_rows = M < kSlabRows ? M : kSlabRows;
+        while (any_rows > 0 && !slab_any_ok(any_rows, lowrank, K, V, mode == 0 ? k : 1, c->sm_count)) any_rows = any_rows > 48 ? 48 : any_rows > 32 ? 32 : any_rows > 16 ? 16 : any_rows > 8 ? 8 : 0;
+    }
+    if (any_rows > 0) {
+        const int pitch = round_up(K, 8);
+        for (int m0 = 0; m0 < M; m0 += any_rows) {
+            const int mrows = M - m0 < any_rows ? M - m0 : any_rows;
+            const bf16* hm = h + (size_t)m0 * d;
+            const bf16* zp[3] = {c->s.zb, c->s.zb_lo, c->s.zb_lo2};
+            if (lowrank) {
+                bf16* const zw[3] = {c->s.zb, c->s.zb_lo, c->s.zb_lo2};
+                CK(stream_code_rows(hm, A, mrows, d, r, pitch, zw, c->sm_count, st));
+                c->launches += 1;
+            } else if (d % 8 == 0 && aligned16(hm)) {
+                zp[0] = hm;
+                zp[1] = zp[2] = nullptr;
+            } else {
+                CK(stream_pad_rows(hm, mrows, d, pitch, c->s.zb, st));
+                zp[1] = zp[2] = nullptr;
+                c->launches += 1;
+            }
+            const bf16* const z[3] = {zp[0], zp[1], zp[2]};
+            CK(slab_head(z, pitch, Bm, mrows, K, V, mode == 0 ? k : 1, mode, mode == 0 ? ids + (size_t)m0 * k : nullptr,
+                         mode == 0 ? logprobs + (size_t)m0 * k : nullptr, mode == 1 ? logits + (size_t)m0 * V : nullptr, c->s, c->sm_count, true, st));
+            c->launches += 1;
+        }
+        return SLIMSPEC_OK;
+    }
+
     if (path == SLIMSPEC_PATH_GENERIC) {
         float* lg = logits;
         if (mode == 0) {
@@ -299,7 +335,8 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
             if (M <= kCodeByStreamRows && d % 2 == 0 && r % 16 == 0) {
                 // few rows: the streaming path's down-projection (one launch of small CTAs) beats a K-split
                 // tcgen05 product plus its reduction
-                e0 = stream_code_rows(h, A, M, d, r, c->s.zb, low_part ? c->s.zb_lo : (bf16*)nullptr, c->sm_count, st);
+                bf16* const zp[3] = {c->s.zb, low_part ? c->s.zb_lo : nullptr, nullptr};
+                e0 = stream_code_rows(h, A, M, d, r, r, zp, c->sm_count, st);
                 n = 1;
             } else {
                 e0 = tensor_downproj(h, A, M, d, r, low_part, c->s, c->sm_count, &n, st);
@@ -338,7 +375,11 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
             // the streaming path's down-projection reads A once per 16 rows: beyond 32 the K-split tensor-core product
             // and its reduction are faster (64 rows, d = 8192, r = 1024: whole call 115.5 us with the one, 81.7 us with the other)
             if (lowrank && mrows > kCodeByStreamRows && d % kTcK == 0 && r >= kTcK) CK(tensor_downproj(hm, A, mrows, d, r, true, c->s, c->sm_count, &nl, st));
-            else if (lowrank) { CK(stream_code_rows(hm, A, mrows, d, r, c->s.zb, c->s.zb_lo, c->sm_count, st)); nl = 1; }
+            else if (lowrank) {
+                bf16* const zp[3] = {c->s.zb, c->s.zb_lo, nullptr};
+                CK(stream_code_rows(hm, A, mrows, d, r, r, zp, c->sm_count, st));
+                nl = 1;
+            }
         } else if (!fma) {
             if (lowrank) CK(stream_code(hm, A, mrows, d, r, V, kk, c->s.zfrag, c->sm_count, st));
             else CK(stream_widen(hm, mrows, d, V, kk, c->s.zfrag, c->sm_count, st));
@@ -362,8 +403,8 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
             CK(fma_head(hm, A, Bm, mrows, fp.mt, d, r, V, kk, mode, ids_t, lp_t, lg_t, c->s, c->epoch, c->sm_count, st));
             nl += 1;
         } else if (use_slab) {
-            CK(slab_head(lowrank ? c->s.zb : hm, lowrank ? c->s.zb_lo : (const bf16*)nullptr, Bm, mrows, K, V, kk, mode, ids_t, lp_t, lg_t, c->s,
-                         c->sm_count, slot < 0, st));
+            const bf16* const zp[3] = {lowrank ? c->s.zb : hm, lowrank ? c->s.zb_lo : nullptr, nullptr};
+            CK(slab_head(zp, K, Bm, mrows, K, V, kk, mode, ids_t, lp_t, lg_t, c->s, c->sm_count, slot < 0, st));
             nl += 1;
         } else {
             int nh = 0;

@@ -16,6 +16,7 @@ struct Scratch {
     uint32_t* zfrag;     // streaming path: the code, as fp32 or as tensor-core fragments (see stream.cu)
     bf16* zb;            // bf16 code [M][r] for the tensor-core path
     bf16* zb_lo;         // its rounding remainder (z - zb), bf16: used while the call is HBM-bound
+    bf16* zb_lo2;        // what the two leave: up to 64 rows, for the shapes that keep all of fp32
     float* zpart;        // K-split partial tiles of the tensor-core down-projection
     size_t zpart_elems;
     uint32_t* smax;      // tensor path: per-row maxima of the sample tiles [64][M padded to 128]
@@ -75,9 +76,11 @@ size_t stream_code_bytes(int K);
 // code = h A for M <= 16 rows, in the form the head kernel for these shapes reads; d even, r a multiple of 16.
 cudaError_t stream_code(const bf16* h, const bf16* A, int M, int d, int r, int V, int k, uint32_t* code, int sm_count,
                         cudaStream_t st);
-// z (bf16, [M][r]) = h A and, if z_lo is not null, its rounding remainder, for any M, on the same kernel:
-// what the tensor-core path uses for small batches instead of a K-split tcgen05 product and a reduction.
-cudaError_t stream_code_rows(const bf16* h, const bf16* A, int M, int d, int r, bf16* z, bf16* z_lo, int sm_count, cudaStream_t st);
+// z = h A for any M and any shape and alignment, on the same kernel, as up to three bf16 matrices [M][pitch] (value,
+// remainder, what the two leave; the later ones may be null).
+cudaError_t stream_code_rows(const bf16* h, const bf16* A, int M, int d, int r, int pitch, bf16* const (&z)[3], int sm_count, cudaStream_t st);
+// dst[M][pitch] = h[M][d]: rows on a pitch that TMA takes.
+cudaError_t stream_pad_rows(const bf16* h, int M, int d, int pitch, bf16* dst, cudaStream_t st);
 // code = h itself (full-rank head: no down-projection).
 cudaError_t stream_widen(const bf16* h, int M, int d, int V, int k, uint32_t* code, int sm_count, cudaStream_t st);
 // logits = z B streamed once (M <= 16); mode 0: fused log-softmax/top-k into ids/logprobs, mode 1: raw logits out.
@@ -85,11 +88,13 @@ cudaError_t stream_head(const uint32_t* code, bool lowrank, const bf16* B, int M
                         int32_t* ids, float* logprobs, float* logits, const Scratch& s, int sm_count,
                         bool after_producer_kernel, int* launches, cudaStream_t st);
 
-// ---- streaming path, three to 64 rows, on the tcgen05 tensor cores (slab.cu) ----------------
+// ---- streaming path, up to 64 rows, on the tcgen05 tensor cores (slab.cu) --------------------
 bool slab_ok(int M, bool lowrank, int K, int V, int k, int sm_count);
+// The same for any V, K and alignment of W (the weights then pass through registers).
+bool slab_any_ok(int M, bool lowrank, int K, int V, int k, int sm_count);
 cudaError_t slab_prepare();
-// logits = z W streamed once; z bf16 [M][K], z_lo (null: z is exact) its rounding remainder.
-cudaError_t slab_head(const bf16* z, const bf16* z_lo, const bf16* W, int M, int K, int V, int k, int mode, int32_t* ids, float* logprobs,
+// logits = z W streamed once; z = z[0] + z[1] + z[2] (null: nothing left) as bf16 [M][K], rows z_pitch elements apart (a multiple of 8).
+cudaError_t slab_head(const bf16* const (&z)[3], int z_pitch, const bf16* W, int M, int K, int V, int k, int mode, int32_t* ids, float* logprobs,
                       float* logits, const Scratch& s, int sm_count, bool pdl, cudaStream_t st);
 
 // ---- the merge of split-V records as a kernel of its own (tensor path; streaming path with many rows)

@@ -78,36 +78,29 @@ __device__ __forceinline__ uint32_t warp_kth_largest64(uint32_t a, uint32_t b, i
     return hit_a ? va : vb;
 }
 
-// A lower bound of the k-th largest (k <= 32 NV) of 32 NV keys, NV per lane, less than 32 NV units of the key below
-// it (the low bits of a key give way to its place, so that the words are distinct and a rank is a plain
-// count).  The words are passed round through s (32 NV of them, of this warp, 16-byte aligned): broadcast
-// reads of four words at a time, where shuffles took four times as long.
+// A lower bound of the k-th largest (k <= 32 NV) of 32 NV keys, NV per lane, by bisection: at least k keys reach it, and
+// no more where a value between the k-th and the next was met, as it nearly always is after eight or ten steps.
+// (Ranks by counting every key against every other took 1000 to 1600 instructions for 128 and 160 keys.)
 template <int NV>
-__device__ __forceinline__ uint32_t warp_kth_bound(const uint32_t (&key)[NV], int k, int lane, uint32_t* s)
+__device__ __forceinline__ uint32_t warp_kth_bisect(const uint32_t (&key)[NV], int k)
 {
-    constexpr uint32_t LOW = NV == 1 ? 31u : NV == 2 ? 63u : NV <= 4 ? 127u : NV <= 8 ? 255u : 511u;
-    uint32_t u[NV];
+    uint32_t mn = key[0], mx = key[0];
 #pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        u[v] = (key[v] & ~LOW) | (LOW - (uint32_t)(lane + 32 * v));
-        s[lane + 32 * v] = u[v];
+    for (int v = 1; v < NV; ++v) { mn = min(mn, key[v]); mx = max(mx, key[v]); }
+    uint32_t lo = warp_min_u32(mn), hi = warp_max_u32(mx) + 1u;       // all keys reach lo, none hi
+    while (hi - lo > 1u) {
+        const uint32_t mid = lo + ((hi - lo) >> 1);
+        int c = 0;
+#pragma unroll
+        for (int v = 0; v < NV; ++v) c += __popc(__ballot_sync(0xffffffffu, key[v] >= mid));
+        if (c >= k) {
+            lo = mid;
+            if (c == k) break;
+        } else {
+            hi = mid;
+        }
     }
-    __syncwarp();
-    int rank[NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) rank[v] = 0;
-#pragma unroll 8
-    for (int i = 0; i < 8 * NV; ++i) {
-        const uint4 o = reinterpret_cast<const uint4*>(s)[i];
-#pragma unroll
-        for (int v = 0; v < NV; ++v) rank[v] += (o.x > u[v]) + (o.y > u[v]) + (o.z > u[v]) + (o.w > u[v]);
-    }
-    uint32_t mine = 0u;          // exactly one of the words has rank k - 1
-#pragma unroll
-    for (int v = 0; v < NV; ++v) mine = rank[v] == k - 1 ? u[v] : mine;
-    const uint32_t r = __reduce_max_sync(0xffffffffu, mine) & ~LOW;
-    __syncwarp();
-    return r;
+    return lo;
 }
 
 // A candidate as one word: larger is better (key descending, id ascending).  0: none.
@@ -168,7 +161,7 @@ __device__ __forceinline__ bool better(uint32_t ka, int ia, uint32_t kb, int ib)
 // (maximum, sum-exp) pairs, written to *lse_out; kind 1 = its k best entries, in order, to out, padded
 // with empty ones (key 0).  A lane owns the records lane, lane + 32, ... (NL of them at most) and keeps what it loads
 // in registers: one round trip to the L2.  area: kMergeWarpBytes of shared memory of this warp, 16-byte aligned.
-static constexpr int kMergeWarpBytes = kMaxRecords * 4 + (kMergeCand + 4) * 8 + 16;
+static constexpr int kMergeWarpBytes = (kMergeCand + 4) * 8 + 16;
 template <int NL>
 __device__ __forceinline__ void merge_task(const float* part, int P, int k, int row, int kind, int lane, float* lse_out,
                                            unsigned long long* out, unsigned char* area)
@@ -192,8 +185,7 @@ __device__ __forceinline__ void merge_task(const float* part, int P, int k, int 
         if (lane == 0) *lse_out = gm + __logf(gs);
         return;
     }
-    uint32_t* s32 = reinterpret_cast<uint32_t*>(area);
-    unsigned long long* cand = reinterpret_cast<unsigned long long*>(s32 + kMaxRecords);
+    unsigned long long* cand = reinterpret_cast<unsigned long long*>(area);
     int* cnt = reinterpret_cast<int*>(cand + kMergeCand + 4);
     // the first three entries of every record, then the bound
     const float2 none = make_float2(0.f, __int_as_float(kNoId));
@@ -212,12 +204,12 @@ __device__ __forceinline__ void merge_task(const float* part, int P, int k, int 
         uint32_t hk[1] = {0u};
 #pragma unroll
         for (int q = 0; q < NL; ++q) hk[0] = max(hk[0], __float_as_uint(e0[q].x));
-        kth = k <= 12 ? warp_kth_rounds(hk[0], k) : warp_kth_bound<1>(hk, k, lane, s32);
+        kth = k <= 12 ? warp_kth_rounds(hk[0], k) : warp_kth_bisect<1>(hk, k);
     } else {
         uint32_t hk[NL];
 #pragma unroll
         for (int q = 0; q < NL; ++q) hk[q] = __float_as_uint(e0[q].x);
-        kth = warp_kth_bound<NL>(hk, k, lane, s32);
+        kth = warp_kth_bisect<NL>(hk, k);
     }
     kth = max(kth, 1u);                      // empty entries (key 0) never count
     // the entries that reach the bound, by ballot: the first ones, then, where any do, the second and third ones (a record's

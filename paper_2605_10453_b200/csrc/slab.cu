@@ -20,6 +20,10 @@
 // tensor memory has room the parts are stacked on the N side (one instruction, two sets of columns,
 // added when the logits are read), else they are two instructions into the same accumulator.
 //
+// Matrices that TMA does not take (a vocabulary that is no multiple of 8, unaligned pointers) come in through registers:
+// warps 2..15 read the aligned 16-byte words around each piece, shift, and store it where TMA would
+// have put it (RAGGED).  The code then has three parts, which is all of fp32.
+//
 // After the stream the logits go row group by row group through shared memory (the ring is idle then), a warp
 // takes a row (maximum, bound below the row's k-th best, sum of exp, candidates, record) and the last CTAs to
 // arrive merge the records (Section 4.1, up-projection; the softmax of Section 3.2; the candidate selection).
@@ -45,15 +49,19 @@ struct alignas(64) SlabParams {
     CUtensorMap mapW;      // W[K][V]: box 64 columns x 32 rows, 128-byte swizzle
     CUtensorMap mapZ;      // code (high part) [M][K]: box 32 columns x zrows rows, 64-byte swizzle
     CUtensorMap mapZ2;     // its remainder, same shape
+    CUtensorMap mapZ3;     // what the two leave
+    const bf16* W;         // ragged: the matrix [K][V]
+    int K;
     int M, V, k, mode;
     int ncta;              // slabs
     int unit_cols, units_base, units_rem;    // slab c has units_base + (c < units_rem) units of unit_cols columns
     int nst, ns;           // stages of the call, stages of the ring
-    int parts, stacked;    // 2: the code comes as value + remainder; 1: stacked on the N side of one instruction
+    int parts, stacked;    // parts the code comes in (1..3); 1: stacked on the N side of one instruction
     int zrows;             // rows of one part in shared memory
     int tcols;             // columns of tensor memory per tile (N of the instruction)
     int tmem_cols;         // columns allocated
     int stage_bytes, wstage_bytes;
+    int raw_off;           // ragged: where the feeders' slots begin, past the ring
     int lpitch;            // floats between two rows of logits in shared memory
     unsigned int idesc;
     int32_t* ids;
@@ -72,12 +80,11 @@ struct alignas(64) SlabParams {
 // instructions and of divergent branches: a version that kept a lane's 56 columns in registers with all loops
 // unrolled took 7900 cycles a row, one that parked candidates as it met them (shared-memory atomics) 5400.
 // area: kSlabRowBytes of shared memory of this warp, 16-byte aligned.
-static constexpr int kSlabRowBytes = 128 * 4 + (kCand + 4) * 8;
+static constexpr int kSlabRowBytes = (kCand + 4) * 8;
 __device__ __forceinline__ void slab_row_record(const float* lr, int nj, int ncols, int col_base, int k, float* part, int row, int P, unsigned char* area, int lane)
 {
     auto rec = [&](int u) -> float2& { return *rec_pair(part, row, P, k, blockIdx.x, u); };
-    uint32_t* s32 = reinterpret_cast<uint32_t*>(area);
-    unsigned long long* cand = reinterpret_cast<unsigned long long*>(s32 + 128);
+    unsigned long long* cand = reinterpret_cast<unsigned long long*>(area);
     const float4* lr4 = reinterpret_cast<const float4*>(lr) + lane;
     float m4[4] = {-FLT_MAX, -FLT_MAX, -FLT_MAX, -FLT_MAX};
 #pragma unroll 2
@@ -94,10 +101,10 @@ __device__ __forceinline__ void slab_row_record(const float* lr, int nj, int nco
         kb = warp_kth_rounds(f2key(lm), k);
     } else if (k <= 32) {
         const uint32_t key[2] = {f2key(fmaxf(m4[0], m4[1])), f2key(fmaxf(m4[2], m4[3]))};
-        kb = warp_kth_bound<2>(key, k, lane, s32);
+        kb = warp_kth_bisect<2>(key, k);
     } else {
         const uint32_t key[4] = {f2key(m4[0]), f2key(m4[1]), f2key(m4[2]), f2key(m4[3])};
-        kb = warp_kth_bound<4>(key, k, lane, s32);
+        kb = warp_kth_bisect<4>(key, k);
     }
     const float cm = warp_max(lm);
     // (Where fewer than k groups hold columns, in a narrow slab, the bound is -FLT_MAX: every column is then a candidate.)
@@ -154,10 +161,111 @@ __device__ __forceinline__ void slab_row_record(const float* lr, int nj, int nco
     __syncwarp();
 }
 
+// Weights through registers (RAGGED).  Rows eight apart are equally far off a 16-byte boundary, whatever V is, so the
+// shift is dealt out by warp: one of the sixteen feeders has a row below 16 and the one 16 further on of every
+// stage and runs one of four loops, each with its shift in words built in.  A step of the loop is 31 pieces of
+// 16 bytes (8 columns) of both rows: the 32 aligned words that cover them come in by cp.async, a word a lane,
+// kSlabSteps steps in flight, each in a slot of its own; then the warp shifts them and stores them where TMA would
+// have.  What counts is the number of instructions (about 20 for 496 bytes; with rows dealt to warps in turn, shift
+// and bounds worked out for each, it was 150, 74 % of the issue slots were busy and the stream ran at 1.0 to 2.0 TB/s)
+// and of loops: with eight, one for each shift in elements, the warps starved for instructions at 0.7 TB/s.
+static constexpr int kSlabSteps = 4;
+static constexpr int kSlabFeeders = 16;
+struct SlabFeed {
+    const bf16* W;
+    int V, K, col0, nu, nst, ns;         // nu: pieces of a row
+    int row0;                            // the warp's first row of a stage; the other is 16 further on
+    uint32_t raw, ring;                  // the lane's word of the warp's first slot; the ring (shared-memory addresses)
+    int stage_bytes;
+    uint64_t *full, *empty;
+    volatile int* abort_flag;
+    int* err;
+};
+
+// The lane's word at q where it need not lie inside the matrix, [beg, end): zeros elsewhere.
+__device__ __noinline__ void slab_feed_edge(uint32_t dst, const char* q, const char* beg, const char* end)
+{
+    if (q >= beg && q + 16 <= end) {
+        asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" ::"r"(dst), "l"(q) : "memory");
+        return;
+    }
+    for (int t = 0; t < 16; t += 2) {
+        const unsigned short w = q + t >= beg && q + t < end ? *reinterpret_cast<const unsigned short*>(q + t) : (unsigned short)0;
+        asm volatile("st.shared.u16 [%0], %1;" ::"r"(dst + t), "h"(w) : "memory");
+    }
+}
+
+template <int WORDS>
+__device__ __forceinline__ void slab_feed(const SlabFeed& f, uint32_t sh)
+{
+    const int lane = threadIdx.x & 31;
+    const int runs = (f.nu + 30) / 31;
+    const char* beg = reinterpret_cast<const char*>(f.W);
+    const char* end = beg + (size_t)f.K * f.V * sizeof(bf16);
+    const long long pitch = 2ll * f.V;
+    const long long down16 = 16 * pitch;
+    const char* q = beg + 2 * (size_t)f.col0 + f.row0 * pitch - 2 * (int)sh + 16 * lane;       // next word to send for, of the first row
+    int qu = 0, qi = 0;
+    auto send = [&](uint32_t dst) {
+        if (qi < f.nst) {
+            if (qi > 0 && (qi + 1) * kSlabStageK < f.K && f.V >= 256) {          // a row away from the matrix's ends
+                asm volatile("cp.async.cg.shared.global [%0], [%1], 16;\n\tcp.async.cg.shared.global [%2], [%3], 16;" ::"r"(dst), "l"(q),
+                             "r"(dst + 512), "l"(q + down16)
+                             : "memory");
+            } else {
+                slab_feed_edge(dst, q, beg, end);
+                slab_feed_edge(dst + 512, q + down16, beg, end);
+            }
+            q += 496;
+            if (++qu == runs) { qu = 0; ++qi; q += 2 * down16 - 496 * runs; }
+        }
+        asm volatile("cp.async.commit_group;" ::: "memory");
+    };
+    for (int d = 0; d < kSlabSteps; ++d) send(f.raw + d * 1024);
+    int s = 0, ph = 0, slot = 0;
+    const uint32_t bits = (sh & 1u) * 16u;
+    const uint32_t x0 = (uint32_t)(f.row0 * 128);            // both rows have the same place modulo 8
+    for (int i = 0; i < f.nst; ++i) {
+        if (i >= f.ns && !mbar_wait_warp(&f.empty[s], ph ^ 1, f.abort_flag, f.err, ERR_WAIT_EMPTY)) break;
+        const uint32_t stage = f.ring + (uint32_t)(s * f.stage_bytes) + x0;
+        for (int u = 0, piece = lane; u < runs; ++u, piece += 31) {
+            asm volatile("cp.async.wait_group %0;" ::"n"(kSlabSteps - 1) : "memory");
+            __syncwarp();
+            const uint32_t src = f.raw + slot * 1024, other = lane < 31 ? 16u : 0u;
+            uint4 a[2], b[2];
+#pragma unroll
+            for (int h = 0; h < 2; ++h) {
+                a[h] = lds128(src + h * 512);
+                b[h] = lds128(src + h * 512 + other);
+            }
+            const uint32_t dst = stage + (uint32_t)((piece >> 3) * kSlabBox + (((piece ^ f.row0) & 7) << 4));
+            if (lane < 31 && piece < f.nu) {
+#pragma unroll
+                for (int h = 0; h < 2; ++h) {
+                    const uint32_t w[8] = {a[h].x, a[h].y, a[h].z, a[h].w, b[h].x, b[h].y, b[h].z, b[h].w};
+                    uint32_t o[4];
+#pragma unroll
+                    for (int j = 0; j < 4; ++j) o[j] = __funnelshift_r(w[j + WORDS], w[j + WORDS + 1], bits);
+                    sts128(dst + h * 2048, o[0], o[1], o[2], o[3]);
+                }
+            }
+            __syncwarp();                                    // everyone has read the slot
+            send(src);
+            slot = (slot + 1) % kSlabSteps;
+        }
+        fence_proxy_async_shared();
+        __syncwarp();
+        if (lane == 0) mbar_arrive(&f.full[s]);
+        if (++s == f.ns) { s = 0; ph ^= 1; }
+    }
+    asm volatile("cp.async.wait_group 0;" ::: "memory");
+}
+
 // RG: rows the tail takes at a time (8, 16 or 32).  At most 112 registers, so that a CTA of the next call's
 // down-projection (128 threads) finds room beside this one.
-template <int RG>
-__global__ void __maxnreg__(112) k_slab_head(const __grid_constant__ SlabParams p)
+static constexpr int kSlabRaggedThreads = kSlabThreads + 64;      // RAGGED: two warps more, so that sixteen feed; the tail is the first sixteen's
+template <int RG, bool RAGGED>
+__global__ void __maxnreg__(RAGGED ? 96 : 112) k_slab_head(const __grid_constant__ SlabParams p)
 {
     extern __shared__ unsigned char smem_raw[];
     __shared__ uint64_t full[kSlabMaxStages], empty[kSlabMaxStages], acc_full;
@@ -175,13 +283,13 @@ __global__ void __maxnreg__(112) k_slab_head(const __grid_constant__ SlabParams 
     const int nbox = (ncols + 63) >> 6, ntile = (nbox + 1) >> 1;
 
     if (tid == 0) {
-        for (int s = 0; s < kSlabMaxStages; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
+        for (int s = 0; s < kSlabMaxStages; ++s) { mbar_init(&full[s], RAGGED ? 1 + kSlabFeeders : 1); mbar_init(&empty[s], 1); }
         mbar_init(&acc_full, 1);
         abort_s = 0;
         mbar_fence_init();
-        prefetch_tensor_map(&p.mapW);
+        if (!RAGGED) prefetch_tensor_map(&p.mapW);
         prefetch_tensor_map(&p.mapZ);
-        if (p.parts == 2) prefetch_tensor_map(&p.mapZ2);
+        if (p.parts >= 2) prefetch_tensor_map(&p.mapZ2);
     }
     if (warp == 1) tmem_alloc(&tmem_base_s, (uint32_t)p.tmem_cols);
     tc_fence_before_sync();
@@ -195,17 +303,19 @@ __global__ void __maxnreg__(112) k_slab_head(const __grid_constant__ SlabParams 
         // code comes from that kernel.
         if (lane == 0) {
             const uint32_t zpart = (uint32_t)p.zrows * 64u;
-            const uint32_t bytes = (uint32_t)nbox * kSlabBox + zpart * (uint32_t)p.parts;
+            const uint32_t bytes = (RAGGED ? 0u : (uint32_t)nbox * kSlabBox) + zpart * (uint32_t)p.parts;
             const int npre = min(p.ns, p.nst);
             auto send_w = [&](int i, int s) {
                 unsigned char* dst = ring + (size_t)s * p.stage_bytes;
                 mbar_arrive_expect_tx(&full[s], bytes);
-                for (int b = 0; b < nbox; ++b) tma_load_2d(dst + b * kSlabBox, &p.mapW, col0 + b * 64, i * kSlabStageK, &full[s]);
+                if (!RAGGED)
+                    for (int b = 0; b < nbox; ++b) tma_load_2d(dst + b * kSlabBox, &p.mapW, col0 + b * 64, i * kSlabStageK, &full[s]);
             };
             auto send_z = [&](int i, int s) {
                 unsigned char* dst = ring + (size_t)s * p.stage_bytes + p.wstage_bytes;
                 tma_load_2d(dst, &p.mapZ, i * kSlabStageK, 0, &full[s]);
-                if (p.parts == 2) tma_load_2d(dst + zpart, &p.mapZ2, i * kSlabStageK, 0, &full[s]);
+                if (p.parts >= 2) tma_load_2d(dst + zpart, &p.mapZ2, i * kSlabStageK, 0, &full[s]);
+                if (p.parts == 3) tma_load_2d(dst + 2 * zpart, &p.mapZ3, i * kSlabStageK, 0, &full[s]);
             };
             for (int i = 0; i < npre; ++i) send_w(i, i);
             pdl_launch_dependents();
@@ -229,7 +339,7 @@ __global__ void __maxnreg__(112) k_slab_head(const __grid_constant__ SlabParams 
             const uint32_t a_lbo = (uint32_t)(kSlabBox >> 4) << 16;                // LBO: the tile's second 64 columns
             const uint32_t stage_w = (uint32_t)p.stage_bytes >> 4, z_off = (uint32_t)p.wstage_bytes >> 4;
             const uint32_t z_part = (uint32_t)(p.zrows * 64) >> 4;
-            const bool two = p.parts == 2 && !p.stacked;
+            const int more = p.stacked ? 0 : p.parts - 1;
             int s = 0, ph = 0;
             bool alive = true;
             for (int i = 0; i < p.nst; ++i) {
@@ -242,7 +352,7 @@ __global__ void __maxnreg__(112) k_slab_head(const __grid_constant__ SlabParams 
                     const uint32_t acc = (i | kk) ? 1u : 0u;
                     for (int t = 0; t < ntile; ++t) {
                         tc_mma_bf16_words2(d, a, A_HI, b, B_HI, p.idesc, acc);
-                        if (two) tc_mma_bf16_words2(d, a, A_HI, b + z_part, B_HI, p.idesc, 1u);
+                        for (int q = 1; q <= more; ++q) tc_mma_bf16_words2(d, a, A_HI, b + (uint32_t)q * z_part, B_HI, p.idesc, 1u);
                         a += (uint32_t)(2 * kSlabBox) >> 4;
                         d += (uint32_t)p.tcols;
                     }
@@ -253,6 +363,30 @@ __global__ void __maxnreg__(112) k_slab_head(const __grid_constant__ SlabParams 
             if (alive) tc_commit(&acc_full);
         }
         __syncwarp();
+    } else if (RAGGED) {
+        // ================= feeders
+        SlabFeed f;
+        f.W = p.W; f.V = p.V; f.K = p.K; f.col0 = col0; f.nu = (ncols + 7) >> 3; f.nst = p.nst; f.ns = p.ns;
+        // Of an odd V the rows' shifts run through all eight values: the four feeders of a scheduler get two shifts that share
+        // a loop (two loops on one scheduler do not fit its instruction buffer: 147 us instead of 95 us for
+        // d = 3072, V = 50257).  Of an even V rows four apart have the same shift, and the plain order does that.
+        if (p.V & 1) {
+            const int n = (warp - 2) >> 2, sh0 = (int)(reinterpret_cast<uintptr_t>(p.W + col0) & 15) >> 1;
+            f.row0 = (((2 * (warp & 3) + (n & 1) - sh0) * p.V) & 7) + 8 * (n >> 1);        // an odd number is its own inverse modulo 8
+        } else {
+            f.row0 = ((warp - 2) & 7) + 8 * ((warp - 2) >> 3);
+        }
+        f.ring = smem_u32(ring);
+        f.raw = f.ring + p.raw_off + (warp - 2) * (kSlabSteps * 1024) + lane * 16;
+        f.stage_bytes = p.stage_bytes;
+        f.full = full; f.empty = empty; f.abort_flag = abort_flag; f.err = p.err;
+        const uint32_t sh = (uint32_t)(reinterpret_cast<uintptr_t>(p.W + (size_t)f.row0 * p.V + col0) & 15) >> 1;
+        switch (sh >> 1) {
+        case 0: slab_feed<0>(f, sh); break;
+        case 1: slab_feed<1>(f, sh); break;
+        case 2: slab_feed<2>(f, sh); break;
+        default: slab_feed<3>(f, sh); break;
+        }
     }
 
     // ================= tail: all warps.  Everything below writes what belongs to the kernels ahead in the stream.
@@ -264,18 +398,20 @@ __global__ void __maxnreg__(112) k_slab_head(const __grid_constant__ SlabParams 
     const int q = warp & 3;                              // the lane quarter of tensor memory this warp may read
     for (int r0 = 0; ok && r0 < p.M; r0 += RG) {
         if (r0 > 0) __syncthreads();                     // the rows before have been worked off
-        for (int t = warp >> 2; t < ntile; t += kSlabThreads / 128) {
+        for (int t = warp >> 2; t < ntile && warp < kSlabThreads / 32; t += kSlabThreads / 128) {
             const uint32_t ta = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(t * p.tcols + r0);
             uint32_t v[RG];
             tmem_ld(ta, v);
+            tmem_ld_wait();
             if (p.stacked) {
-                uint32_t w[RG];
-                tmem_ld(ta + (uint32_t)p.zrows, w);
-                tmem_ld_wait();
+#pragma unroll 1
+                for (int part = 1; part < p.parts; ++part) {
+                    uint32_t w[RG];
+                    tmem_ld(ta + (uint32_t)(part * p.zrows), w);
+                    tmem_ld_wait();
 #pragma unroll
-                for (int n = 0; n < RG; ++n) v[n] = __float_as_uint(__uint_as_float(v[n]) + __uint_as_float(w[n]));
-            } else {
-                tmem_ld_wait();
+                    for (int n = 0; n < RG; ++n) v[n] = __float_as_uint(__uint_as_float(v[n]) + __uint_as_float(w[n]));
+                }
             }
             const int c = t * 128 + q * 32 + lane;
             if (p.mode == 0) {
@@ -290,7 +426,7 @@ __global__ void __maxnreg__(112) k_slab_head(const __grid_constant__ SlabParams 
         if (p.mode == 0) {
             __syncthreads();
             const int rows = min(RG, p.M - r0);
-            for (int n = warp; n < rows; n += kSlabThreads / 32) {
+            for (int n = warp; n < rows && warp < kSlabThreads / 32; n += kSlabThreads / 32) {
                 const float* lr = lg + (size_t)n * p.lpitch;
                 slab_row_record(lr, ntile, ncols, col0, p.k, p.part, r0 + n, p.ncta, row_area, lane);
             }
@@ -306,13 +442,15 @@ __global__ void __maxnreg__(112) k_slab_head(const __grid_constant__ SlabParams 
 // ------------------------------------------------------------------------------------------
 struct SlabGeometry {
     int ncta, unit_cols, units_base, units_rem, ntile, ns, rg;
-    int zrows, stacked, tcols, tmem_cols, stage_bytes, wstage_bytes, lpitch;
+    int zrows, stacked, tcols, tmem_cols, stage_bytes, wstage_bytes, raw_off, lpitch;
     size_t smem;
 };
 
-static bool slab_geometry(int M, int parts, int K, int V, int k, int sm_count, SlabGeometry* g)
+// Everything but the layout of W: M <= 64, k <= 64.
+static bool slab_geometry(int M, int parts, int K, int V, int k, int sm_count, bool ragged, SlabGeometry* g)
 {
-    if (M < 1 || M > 64 || V % 8 != 0 || V < 64 || K < 8 || K % 8 != 0 || k < 1 || k > kMaxK) return false;
+    if (M < 1 || M > 64 || V < 1 || K < 1 || k < 1 || k > kMaxK) return false;
+    const int warps = (ragged ? kSlabRaggedThreads : kSlabThreads) / 32;
     // Slabs start on a 128-byte line while that costs little balance; narrow slabs (small vocabularies)
     // are cut finer.
     int uc = 64;
@@ -328,9 +466,9 @@ static bool slab_geometry(int M, int parts, int K, int V, int k, int sm_count, S
     if (g->ntile > kSlabMaxTiles) return false;
     g->rg = M <= 8 ? 8 : (M <= 16 || (M > 32 && M <= 48)) ? 16 : 32;      // rows of the tail's groups; 33..48 rows: three groups of 16
     const int mpad = (M + g->rg - 1) / g->rg * g->rg;
-    g->zrows = parts == 2 ? mpad : (mpad < 16 ? 16 : mpad);
-    g->stacked = parts == 2 && (g->ntile * 2 * g->zrows <= 512 || g->zrows < 16) ? 1 : 0;
-    g->tcols = g->stacked ? 2 * g->zrows : g->zrows;
+    g->zrows = parts == 2 ? mpad : (mpad < 16 ? 16 : mpad);             // N of an instruction is a multiple of 16
+    g->stacked = parts > 1 && (g->ntile * parts * g->zrows <= 512 || g->zrows < 16) ? 1 : 0;
+    g->tcols = g->stacked ? parts * g->zrows : g->zrows;
     if (g->ntile * g->tcols > 512) return false;
     g->tmem_cols = 32;
     while (g->tmem_cols < g->ntile * g->tcols) g->tmem_cols *= 2;
@@ -341,57 +479,79 @@ static bool slab_geometry(int M, int parts, int K, int V, int k, int sm_count, S
     if (ns > kSlabMaxStages) ns = kSlabMaxStages;
     g->ns = ns;
     g->lpitch = g->ntile * 128;
-    size_t area = (size_t)ns * g->stage_bytes;
+    g->raw_off = ns * g->stage_bytes;
+    size_t area = (size_t)g->raw_off + (ragged ? (size_t)kSlabFeeders * kSlabSteps * 1024 : 0);
     const size_t tail = (size_t)g->rg * g->lpitch * 4 + (size_t)(kSlabThreads / 32) * kSlabRowBytes;
     if (area < tail) area = tail;
     // the merge: R CTAs share the rows
-    int R = (M + 7) / 8;
+    int R = (M + warps / 2 - 1) / (warps / 2);
     if (R > g->ncta) R = g->ncta;
     const int mine = (M + R - 1) / R;
     if (mine > 16) return false;
-    if (area < (size_t)merge_area_bytes(mine, kSlabThreads / 32)) area = merge_area_bytes(mine, kSlabThreads / 32);
+    if (area < (size_t)merge_area_bytes(mine, warps)) area = merge_area_bytes(mine, warps);
     g->smem = 1024 + area;
     return g->smem <= kSlabSmemMax;
 }
 
+// W as TMA takes it (rows of a multiple of 16 bytes; the pointer is the caller's to check), and the code likewise.
 bool slab_ok(int M, bool lowrank, int K, int V, int k, int sm_count)
 {
     SlabGeometry g;
-    return slab_geometry(M, lowrank ? 2 : 1, K, V, k, sm_count, &g);
+    return V % 8 == 0 && V >= 64 && K >= 8 && K % 8 == 0 && slab_geometry(M, lowrank ? 2 : 1, K, V, k, sm_count, false, &g);
 }
+
+// Any V and K, any alignment of W.
+bool slab_any_ok(int M, bool lowrank, int K, int V, int k, int sm_count)
+{
+    SlabGeometry g;
+    return slab_geometry(M, lowrank ? 3 : 1, K, V, k, sm_count, true, &g);
+}
+
+template <typename Kern>
+static cudaError_t slab_allow(Kern kern) { return cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSlabSmemMax); }
 
 cudaError_t slab_prepare()
 {
     cudaError_t e;
-    if ((e = cudaFuncSetAttribute(k_slab_head<8>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSlabSmemMax)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_slab_head<16>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSlabSmemMax)) != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_slab_head<32>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kSlabSmemMax);
+    if ((e = slab_allow(k_slab_head<8, false>)) != cudaSuccess || (e = slab_allow(k_slab_head<8, true>)) != cudaSuccess) return e;
+    if ((e = slab_allow(k_slab_head<16, false>)) != cudaSuccess || (e = slab_allow(k_slab_head<16, true>)) != cudaSuccess) return e;
+    if ((e = slab_allow(k_slab_head<32, false>)) != cudaSuccess) return e;
+    return slab_allow(k_slab_head<32, true>);
 }
 
-cudaError_t slab_head(const bf16* z, const bf16* z_lo, const bf16* W, int M, int K, int V, int k, int mode, int32_t* ids, float* logprobs,
+template <int RG, bool RAGGED>
+static cudaError_t slab_launch(const SlabGeometry& g, bool pdl, cudaStream_t st, const SlabParams& p)
+{
+    return launch_chain(k_slab_head<RG, RAGGED>, g.ncta, RAGGED ? kSlabRaggedThreads : kSlabThreads, g.smem, pdl, st, p);
+}
+
+cudaError_t slab_head(const bf16* const (&z)[3], int z_pitch, const bf16* W, int M, int K, int V, int k, int mode, int32_t* ids, float* logprobs,
                       float* logits, const Scratch& s, int sm_count, bool pdl, cudaStream_t st)
 {
     SlabGeometry g;
-    const int parts = z_lo != nullptr ? 2 : 1;
-    if (!slab_geometry(M, parts, K, V, k, sm_count, &g)) return cudaErrorInvalidValue;
+    const int parts = z[2] != nullptr ? 3 : z[1] != nullptr ? 2 : 1;
+    const bool ragged = V % 8 != 0 || V < 64 || ((uintptr_t)W & 15) != 0;
+    if (!slab_geometry(M, parts, K, V, k, sm_count, ragged, &g)) return cudaErrorInvalidValue;
     SlabParams p;
     memset(&p, 0, sizeof(p));
-    if (!make_map(&p.mapW, W, K, V, 64, kSlabStageK) || !make_map(&p.mapZ, z, M, K, 32, g.zrows)) return cudaErrorInvalidValue;
-    if (parts == 2 && !make_map(&p.mapZ2, z_lo, M, K, 32, g.zrows)) return cudaErrorInvalidValue;
+    if (!ragged && !make_map(&p.mapW, W, K, V, 64, kSlabStageK)) return cudaErrorInvalidValue;
+    CUtensorMap* mz[3] = {&p.mapZ, &p.mapZ2, &p.mapZ3};
+    for (int q = 0; q < parts; ++q)
+        if (!make_map_pitched(mz[q], z[q], M, K, z_pitch, 32, g.zrows)) return cudaErrorInvalidValue;
+    p.W = W; p.K = K;
     p.M = M; p.V = V; p.k = k; p.mode = mode;
     p.ncta = g.ncta; p.unit_cols = g.unit_cols; p.units_base = g.units_base; p.units_rem = g.units_rem;
     p.nst = (K + kSlabStageK - 1) / kSlabStageK; p.ns = g.ns;
     p.parts = parts; p.stacked = g.stacked; p.zrows = g.zrows; p.tcols = g.tcols; p.tmem_cols = g.tmem_cols;
-    p.stage_bytes = g.stage_bytes; p.wstage_bytes = g.wstage_bytes; p.lpitch = g.lpitch;
+    p.stage_bytes = g.stage_bytes; p.wstage_bytes = g.wstage_bytes; p.raw_off = g.raw_off; p.lpitch = g.lpitch;
     // D fp32, A and B bf16, A MN-major, B K-major, N = columns of a tile, M = 128
     p.idesc = (1u << 4) | (1u << 7) | (1u << 10) | (1u << 15) | ((uint32_t)(g.tcols >> 3) << 17) | (8u << 24);
     p.ids = ids; p.logprobs = logprobs; p.logits = logits;
     p.part = s.part; p.ticket = s.tickets; p.err = s.err;
     p.ticket_base = mode == 0 ? *s.ticket_base_host : 0u;
     if (mode == 0 && (size_t)M * 2 * rec_row_pairs(p.ncta, k) > s.part_elems) return cudaErrorInvalidValue;
-    const cudaError_t e = g.rg == 8 ? launch_chain(k_slab_head<8>, g.ncta, kSlabThreads, g.smem, pdl, st, p)
-                        : g.rg == 16 ? launch_chain(k_slab_head<16>, g.ncta, kSlabThreads, g.smem, pdl, st, p)
-                                     : launch_chain(k_slab_head<32>, g.ncta, kSlabThreads, g.smem, pdl, st, p);
+    const cudaError_t e = ragged ? (g.rg == 8 ? slab_launch<8, true>(g, pdl, st, p) : g.rg == 16 ? slab_launch<16, true>(g, pdl, st, p) : slab_launch<32, true>(g, pdl, st, p))
+                        : g.rg == 8 ? slab_launch<8, false>(g, pdl, st, p) : g.rg == 16 ? slab_launch<16, false>(g, pdl, st, p) : slab_launch<32, false>(g, pdl, st, p);
     if (e == cudaSuccess && mode == 0) *s.ticket_base_host += (unsigned int)p.ncta;      // the tickets this launch will take
     return e;
 }

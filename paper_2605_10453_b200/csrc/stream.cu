@@ -128,8 +128,8 @@ struct CodeParams {
     int nbuf;         // buffers
     int fmt;          // kCodePacked, kCodeSplit or kCodeRows
     uint32_t* zfrag;  // the code in that form
-    bf16* zrows;      // kCodeRows: value [M][r]
-    bf16* zrows_lo;   // kCodeRows: remainder [M][r], or null
+    bf16* zrows[3];   // kCodeRows: value, remainder and what the two leave, [M][pitch]; the later ones may be null
+    int pitch;
 };
 
 static constexpr int kCodePitch = 80;            // bytes between two rows of the A slice in shared memory: 5 units (odd)
@@ -139,6 +139,8 @@ static constexpr int kCodeChunkRows = 320;       // ... else it works through it
 static constexpr int kCodeRing = 4;              // through a ring of this many buffers, two CTAs per SM
 static constexpr size_t kCodeSmemMax = (size_t)kCodeRing * kCodeChunkRows * kCodePitch + 128;   // most dynamic shared memory of that kernel
 
+// PLAIN: any d, r and alignment (element by element); else d even, r a multiple of 8, A 16-byte and h 4-byte aligned.
+template <bool PLAIN>
 __global__ void __launch_bounds__(128, 8) k_stream_code(const CodeParams p)
 {
     __shared__ __align__(16) float wt[4][16 * 32];      // the warps' partial tiles
@@ -165,6 +167,16 @@ __global__ void __launch_bounds__(128, 8) k_stream_code(const CodeParams p)
             const int kb0 = cta_kb0 + c * chunk_kbs, kb1 = min(cta_kb1, kb0 + chunk_kbs);
             unsigned char* dst = aslice + (size_t)(c % nbuf) * buf_bytes;
             const int rows = 16 * (kb1 - kb0);
+            if (PLAIN) {
+#pragma unroll 4
+                for (int idx = tid; idx < rows * 16; idx += 128) {
+                    const int row = idx >> 4, c2 = (idx & 15) * 2;
+                    const bf16* src = p.A + (size_t)min(16 * kb0 + row, d - 1) * r;
+                    const uint32_t x = __bfloat16_as_ushort(src[min(j0 + c2, r - 1)]), y = __bfloat16_as_ushort(src[min(j0 + c2 + 1, r - 1)]);
+                    *reinterpret_cast<uint32_t*>(dst + (size_t)row * kCodePitch + c2 * 2) = x | (y << 16);
+                }
+                return;
+            }
             for (int idx = tid; idx < rows * 4; idx += 128) {
                 const int row = idx >> 2, u = idx & 3;
                 const int grow = min(16 * kb0 + row, d - 1);             // rows past d re-read the last row (their h is zero)
@@ -201,6 +213,16 @@ __global__ void __launch_bounds__(128, 8) k_stream_code(const CodeParams p)
                 const int k0 = 16 * (kb + i) + 2 * t;
                 const bool on = kb + i < wb1;
                 const bool lo_ok = on && k0 < d, hi_ok = on && k0 + 8 < d;
+                if (PLAIN) {
+                    auto pair = [&](int row, int kk) -> uint32_t {
+                        uint32_t w = 0u;
+                        if (on && row < mrows && kk < d) w = __bfloat16_as_ushort(hrows[(size_t)row * d + kk]);
+                        if (on && row < mrows && kk + 1 < d) w |= (uint32_t)__bfloat16_as_ushort(hrows[(size_t)row * d + kk + 1]) << 16;
+                        return w;
+                    };
+                    hf[i] = make_uint4(pair(g, k0), pair(g + 8, k0), pair(g, k0 + 8), pair(g + 8, k0 + 8));
+                    continue;
+                }
                 const uint32_t* h0 = reinterpret_cast<const uint32_t*>(hrows + (size_t)g * d + k0);
                 const uint32_t* h1 = reinterpret_cast<const uint32_t*>(hrows + (size_t)(g + 8) * d + k0);
                 hf[i].x = (g < mrows && lo_ok) ? __ldcg(h0) : 0u;
@@ -258,19 +280,22 @@ __global__ void __launch_bounds__(128, 8) k_stream_code(const CodeParams p)
     const int row = tid >> 3, j = j0 + (tid & 7) * 4;
     if (j >= r) return;
     const float z[4] = {v.x, v.y, v.z, v.w};
-    uint32_t hi[4], lo[4];
+    uint32_t hi[4], lo[4], lo2[4];
 #pragma unroll
     for (int e = 0; e < 4; ++e) {
         const bf16 hb = __float2bfloat16_rn(z[e]);
-        const bf16 lb = __float2bfloat16_rn(z[e] - __bfloat162float(hb));
+        const float rest = z[e] - __bfloat162float(hb);
+        const bf16 lb = __float2bfloat16_rn(rest);
         hi[e] = (uint32_t)__bfloat16_as_ushort(hb);
         lo[e] = (uint32_t)__bfloat16_as_ushort(lb);
+        lo2[e] = (uint32_t)__bfloat16_as_ushort(__float2bfloat16_rn(rest - __bfloat162float(lb)));
     }
     if (p.fmt == kCodeRows) {
         if (row < mrows) {
-            const size_t o = (size_t)(m0 + row) * r + j;          // four bf16: 8 bytes, aligned (j is a multiple of 4)
-            *reinterpret_cast<uint2*>(p.zrows + o) = make_uint2(hi[0] | (hi[1] << 16), hi[2] | (hi[3] << 16));
-            if (p.zrows_lo) *reinterpret_cast<uint2*>(p.zrows_lo + o) = make_uint2(lo[0] | (lo[1] << 16), lo[2] | (lo[3] << 16));
+            const size_t o = (size_t)(m0 + row) * p.pitch + j;     // four bf16: 8 bytes, aligned (j and the pitch are multiples of 4; past r there is room to the pitch)
+            *reinterpret_cast<uint2*>(p.zrows[0] + o) = make_uint2(hi[0] | (hi[1] << 16), hi[2] | (hi[3] << 16));
+            if (p.zrows[1]) *reinterpret_cast<uint2*>(p.zrows[1] + o) = make_uint2(lo[0] | (lo[1] << 16), lo[2] | (lo[3] << 16));
+            if (p.zrows[2]) *reinterpret_cast<uint2*>(p.zrows[2] + o) = make_uint2(lo2[0] | (lo2[1] << 16), lo2[2] | (lo2[3] << 16));
         }
         return;
     }
@@ -306,6 +331,16 @@ __global__ void k_stream_widen(const bf16* __restrict__ h, int M, int d, int nkb
     zfrag[w] = word;
 }
 
+
+__global__ void k_stream_pad_rows(const bf16* __restrict__ h, int M, int d, int pitch, bf16* __restrict__ dst)
+{
+    pdl_launch_dependents();
+    pdl_wait();
+    const int i = blockIdx.x * blockDim.x + threadIdx.x;
+    if (i >= M * pitch) return;
+    const int m = i / pitch, c = i - m * pitch;
+    dst[i] = c < d ? h[(size_t)m * d + c] : __float2bfloat16_rn(0.f);
+}
 
 // ------------------------------------------------------------------------------------------
 // Three to sixteen rows.  One CTA per V slab, seven warps, two CTAs per SM: all warps of a CTA meet
@@ -566,7 +601,7 @@ static bool plan_code(int M, bool lowrank, int K, int V, int k, int sm_count, Ge
 // before it in the stream has signalled launch_dependents or left; it orders itself after that
 // kernel with griddepcontrol.wait.  Across calls this hides the launch gap and lets the first
 // kernel of a call warm up under the tail of the last kernel of the call before.
-static cudaError_t launch_code(CodeParams cp, int sm_count, size_t head_smem, cudaStream_t st)
+static cudaError_t launch_code(CodeParams cp, bool plain, int sm_count, size_t head_smem, cudaStream_t st)
 {
     cp.nkb = (cp.d + 15) / 16;
     const int nct = (cp.r + 31) / 32;
@@ -614,7 +649,7 @@ static cudaError_t launch_code(CodeParams cp, int sm_count, size_t head_smem, cu
     attr[1].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 2;
-    return cudaLaunchKernelEx(&cfg, k_stream_code, cp);
+    return plain ? cudaLaunchKernelEx(&cfg, k_stream_code<true>, cp) : cudaLaunchKernelEx(&cfg, k_stream_code<false>, cp);
 }
 
 cudaError_t stream_code(const bf16* h, const bf16* A, int M, int d, int r, int V, int k, uint32_t* zfrag, int sm_count,
@@ -625,17 +660,33 @@ cudaError_t stream_code(const bf16* h, const bf16* A, int M, int d, int r, int V
     memset(&cp, 0, sizeof(cp));
     if (!plan_code(M, true, r, V, k, sm_count, &g, &cp.fmt)) return cudaErrorInvalidValue;
     cp.h = h; cp.A = A; cp.M = M; cp.d = d; cp.r = r; cp.zfrag = zfrag;
-    return launch_code(cp, sm_count, g.smem, st);
+    return launch_code(cp, false, sm_count, g.smem, st);
 }
 
-cudaError_t stream_code_rows(const bf16* h, const bf16* A, int M, int d, int r, bf16* z, bf16* z_lo, int sm_count, cudaStream_t st)
+cudaError_t stream_code_rows(const bf16* h, const bf16* A, int M, int d, int r, int pitch, bf16* const (&z)[3], int sm_count, cudaStream_t st)
 {
-    if (d % 2 != 0 || r % 16 != 0 || M < 1) return cudaErrorInvalidValue;
+    if (M < 1 || pitch % 4 != 0 || pitch < r) return cudaErrorInvalidValue;
     CodeParams cp;
     memset(&cp, 0, sizeof(cp));
     cp.fmt = kCodeRows;
-    cp.h = h; cp.A = A; cp.M = M; cp.d = d; cp.r = r; cp.zrows = z; cp.zrows_lo = z_lo;
-    return launch_code(cp, sm_count, 0, st);
+    cp.h = h; cp.A = A; cp.M = M; cp.d = d; cp.r = r; cp.pitch = pitch;
+    for (int q = 0; q < 3; ++q) cp.zrows[q] = z[q];
+    const bool plain = d % 2 != 0 || r % 8 != 0 || ((uintptr_t)A & 15) != 0 || ((uintptr_t)h & 3) != 0;
+    return launch_code(cp, plain, sm_count, 0, st);
+}
+
+cudaError_t stream_pad_rows(const bf16* h, int M, int d, int pitch, bf16* dst, cudaStream_t st)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((M * pitch + 255) / 256);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k_stream_pad_rows, h, M, d, pitch, dst);
 }
 
 cudaError_t stream_widen(const bf16* h, int M, int d, int V, int k, uint32_t* zfrag, int sm_count, cudaStream_t st)
@@ -669,8 +720,9 @@ cudaError_t stream_prepare()
 {
     cudaError_t e;
     cudaFuncAttributes fa;
-    if ((e = cudaFuncGetAttributes(&fa, k_stream_code)) != cudaSuccess) return e;
-    if ((e = cudaFuncSetAttribute(k_stream_code, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCodeSmemMax)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_stream_code<false>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCodeSmemMax)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_stream_code<true>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kCodeSmemMax)) != cudaSuccess) return e;
+    if ((e = cudaFuncGetAttributes(&fa, k_stream_pad_rows)) != cudaSuccess) return e;
     if ((e = cudaFuncGetAttributes(&fa, k_stream_widen)) != cudaSuccess) return e;
     if ((e = allow_smem(k_stream_head_mma<8, 1, 1>)) != cudaSuccess) return e;
     if ((e = allow_smem(k_stream_head_mma<8, 1, 2>)) != cudaSuccess) return e;
