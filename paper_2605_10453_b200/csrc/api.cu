@@ -37,7 +37,6 @@ static const int kTimingEvents = 256;
 static const int kMaxParts = 320;      // most split-V records any kernel writes per row
 static const int kStreamMaxRows = 16;  // largest M the streaming path is chosen for
 static const int kSplitCodeRows = 256;  // tensor path: z carried as hi + lo bf16 parts while the call is HBM-bound (up to this many rows)
-static const int kTcK = 64;             // the tensor-core down-projection: d a multiple of this, r at least this
 static const int kRowPad = 8;          // rows of the generic path's fp32 code are padded to this
 static const int kStreamTile = 16;     // rows one launch of the older streaming kernels takes
 static const int kSlabRows = 64;       // rows one launch of the slab kernel takes
@@ -85,23 +84,17 @@ extern "C" int slimspec_create(slimspec_ctx** out, int max_M, int max_d, int max
     const size_t mpad128 = (size_t)round_up(max_M, 128);
     const size_t part_elems = ((size_t)kStreamTile * kMaxParts + (size_t)(c->sm_count + 12) * 256 + 2 * mpad128) *
                               (size_t)(2 + 2 * rec_k);
-    // K-split partial tiles of the tensor-core down-projection: one 128 x 128 fp32 tile per SM, or one split
-    size_t zpart_elems = (size_t)(c->sm_count + 12) * 128 * 128;
-    if (zpart_elems < mpad128 * (size_t)max_d) zpart_elems = mpad128 * (size_t)max_d;
     bool ok = true;
     ok = ok && cudaMalloc(&c->s.z, z_elems * sizeof(float)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->s.part, part_elems * sizeof(float)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->s.zfrag, stream_code_bytes(max_d)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->s.zq, fma_code_words(max_d) * sizeof(uint2)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->s.zpart, zpart_elems * sizeof(float)) == cudaSuccess;
     const size_t dpad = (size_t)round_up(max_d, 8);          // rows on a pitch that TMA takes
     ok = ok && cudaMalloc(&c->s.zb, (2 * mpad128 + kSlabRows) * dpad * sizeof(bf16)) == cudaSuccess;
     if (ok) { c->s.zb_lo = c->s.zb + mpad128 * dpad; c->s.zb_lo2 = c->s.zb_lo + mpad128 * dpad; }
-    ok = ok && cudaMalloc(&c->s.smax, 64 * mpad128 * sizeof(uint32_t)) == cudaSuccess;
-    ok = ok && cudaMalloc(&c->s.thr0, mpad128 * sizeof(uint32_t)) == cudaSuccess;
-    c->s.smax_elems = 64 * mpad128;
+    ok = ok && cudaMalloc(&c->s.bound, 32 * mpad128 * sizeof(unsigned long long)) == cudaSuccess;
+    c->s.bound_pitch = (int)mpad128;
     c->s.part_elems = part_elems;
-    c->s.zpart_elems = zpart_elems;
     ok = ok && cudaMalloc(&c->s.tickets, 4096 * sizeof(unsigned int)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->s.err, sizeof(int)) == cudaSuccess;
     ok = ok && cudaMalloc(&c->h_stage, (size_t)max_M * max_d * sizeof(bf16)) == cudaSuccess;
@@ -120,7 +113,8 @@ extern "C" int slimspec_create(slimspec_ctx** out, int max_M, int max_d, int max
     ok = ok && cudaMemset(c->s.err, 0, sizeof(int)) == cudaSuccess;
     ok = ok && cudaMemset(c->s.zq, 0, fma_code_words(max_d) * sizeof(uint2)) == cudaSuccess;
     ok = ok && cudaMemset(c->s.z, 0, z_elems * sizeof(float)) == cudaSuccess;
-    ok = ok && stream_prepare() == cudaSuccess && slab_prepare() == cudaSuccess && fma_prepare() == cudaSuccess;
+    ok = ok && cudaMemset(c->s.bound, 0, 32 * mpad128 * sizeof(unsigned long long)) == cudaSuccess;
+    ok = ok && stream_prepare() == cudaSuccess && slab_prepare() == cudaSuccess && tensor_prepare() == cudaSuccess && fma_prepare() == cudaSuccess;
     ok = ok && cudaDeviceSynchronize() == cudaSuccess;
     if (!ok) {
         cudaGetLastError();
@@ -135,7 +129,7 @@ extern "C" void slimspec_destroy(slimspec_ctx* c)
 {
     if (!c) return;
     cudaDeviceSynchronize();
-    cudaFree(c->s.z); cudaFree(c->s.zfrag); cudaFree(c->s.zq); cudaFree(c->s.part); cudaFree(c->s.zpart); cudaFree(c->s.zb); cudaFree(c->s.smax); cudaFree(c->s.thr0); cudaFree(c->s.tickets); cudaFree(c->s.err);
+    cudaFree(c->s.z); cudaFree(c->s.zfrag); cudaFree(c->s.zq); cudaFree(c->s.part); cudaFree(c->s.zb); cudaFree(c->s.bound); cudaFree(c->s.tickets); cudaFree(c->s.err);
     cudaFree(c->s.logits); cudaFree(c->h_stage);
     if (c->res_host) cudaFreeHost(c->res_host);
     if (c->ev0) {
@@ -238,6 +232,19 @@ static int ensure_logits(slimspec_ctx* c, size_t elems)
 
 #define CK(expr) do { if ((expr) != cudaSuccess) { cudaGetLastError(); return SLIMSPEC_ERR_CUDA; } } while (0)
 
+// The number of the next call.  When the numbers have gone round, what carries the old ones is forgotten.
+static cudaError_t next_epoch(slimspec_ctx* c, cudaStream_t st, unsigned int* epoch)
+{
+    cudaError_t e = cudaSuccess;
+    if (++c->epoch == 0) {
+        e = cudaMemsetAsync(c->s.zq, 0, fma_code_words(c->max_d) * sizeof(uint2), st);
+        if (e == cudaSuccess) e = cudaMemsetAsync(c->s.bound, 0, (size_t)32 * c->s.bound_pitch * sizeof(unsigned long long), st);
+        c->epoch = 1;
+    }
+    *epoch = c->epoch;
+    return e;
+}
+
 // Shared body.  K is the contraction length of the streamed matrix Bm (K x V): r for the
 // low-rank head (A != null), d for the full-rank head (A == null, z = widened h).
 // mode 0: top-k into ids/logprobs; mode 1: raw logits.
@@ -263,7 +270,7 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
     const bool slab = ptr_ok && d % 2 == 0 && (!lowrank || r % 16 == 0) && slab_ok(slab_rows, lowrank, K, V, mode == 0 ? k : 1, c->sm_count) &&
                       !(mode == 1 && M <= kStreamMaxRows && sp.ok);
     const bool stream_ok = (slab && k <= 32) || (sp.ok && ptr_ok && d % 2 == 0 && (!lowrank || r % 16 == 0));
-    const bool tensor_fits = tensor_ok(M, K, V, k, mode) && ptr_ok && (!lowrank || (d % kTcK == 0 && r >= kTcK));
+    const bool tensor_fits = tensor_ok(M, lowrank, K, V, k, mode) && ptr_ok;
     if (path == SLIMSPEC_PATH_AUTO) {
         // FP32 FMAs keep up with HBM only for a few rows; beyond that the tensor cores take over
         if (M > (slab ? kSlabRows : kStreamMaxRows) && tensor_fits) path = SLIMSPEC_PATH_TENSOR;
@@ -327,19 +334,19 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
         int n = 0;
         const bf16* X = h;
         const bf16* Xlo = nullptr;
+        const int x_pitch = round_up(K, 8);
         if (lowrank) {
             // While the call is HBM-bound the tensor cores have time to spare: keep the bf16 rounding
             // remainder of z and feed it through a second MMA, so z is effectively fp32-exact.
             const bool low_part = M <= kSplitCodeRows;
             cudaError_t e0;
-            if (M <= kCodeByStreamRows && d % 2 == 0 && r % 16 == 0) {
-                // few rows: the streaming path's down-projection (one launch of small CTAs) beats a K-split
-                // tcgen05 product plus its reduction
-                bf16* const zp[3] = {c->s.zb, low_part ? c->s.zb_lo : nullptr, nullptr};
-                e0 = stream_code_rows(h, A, M, d, r, r, zp, c->sm_count, st);
-                n = 1;
+            if (M > kCodeByStreamRows && tensor_code_ok(d, r)) {
+                e0 = tensor_downproj(h, A, M, d, r, c->s.zb, low_part ? c->s.zb_lo : nullptr, x_pitch, c->s, c->sm_count, &n, st);
             } else {
-                e0 = tensor_downproj(h, A, M, d, r, low_part, c->s, c->sm_count, &n, st);
+                // few rows: the streaming path's down-projection (one launch of small CTAs) is the faster one; it also takes every shape
+                bf16* const zp[3] = {c->s.zb, low_part ? c->s.zb_lo : nullptr, nullptr};
+                e0 = stream_code_rows(h, A, M, d, r, x_pitch, zp, c->sm_count, st);
+                n = 1;
             }
             c->launches += n;
             n = 0;
@@ -353,7 +360,9 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
             if (c->timing_used == kTimingEvents) { int rc = timing_drain(c); if (rc != SLIMSPEC_OK) return rc; }
             slot = c->timing_used++;
         }
-        cudaError_t e = tensor_head(X, Xlo, Bm, M, K, V, k, mode, ids, logprobs, logits, c->s, c->sm_count, &n,
+        unsigned int epoch = 0;
+        CK(next_epoch(c, st, &epoch));
+        cudaError_t e = tensor_head(X, Xlo, x_pitch, Bm, M, K, V, k, mode, ids, logprobs, logits, c->s, epoch, c->sm_count, &n,
                                     slot >= 0 ? c->ev0[slot] : (cudaEvent_t) nullptr, slot >= 0 ? c->ev1[slot] : (cudaEvent_t) nullptr, st);
         c->launches += n;
         if (e != cudaSuccess) { cudaGetLastError(); return SLIMSPEC_ERR_CUDA; }
@@ -374,7 +383,7 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
         if (use_slab) {
             // the streaming path's down-projection reads A once per 16 rows: beyond 32 the K-split tensor-core product
             // and its reduction are faster (64 rows, d = 8192, r = 1024: whole call 115.5 us with the one, 81.7 us with the other)
-            if (lowrank && mrows > kCodeByStreamRows && d % kTcK == 0 && r >= kTcK) CK(tensor_downproj(hm, A, mrows, d, r, true, c->s, c->sm_count, &nl, st));
+            if (lowrank && mrows > kCodeByStreamRows && tensor_code_ok(d, r)) CK(tensor_downproj(hm, A, mrows, d, r, c->s.zb, c->s.zb_lo, r, c->s, c->sm_count, &nl, st));
             else if (lowrank) {
                 bf16* const zp[3] = {c->s.zb, c->s.zb_lo, nullptr};
                 CK(stream_code_rows(hm, A, mrows, d, r, r, zp, c->sm_count, st));
@@ -396,11 +405,9 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
         float* lp_t = mode == 0 ? logprobs + (size_t)m0 * k : nullptr;
         float* lg_t = mode == 1 ? logits + (size_t)m0 * V : nullptr;
         if (fma) {
-            if (++c->epoch == 0) {      // the call numbers have gone round: forget the old ones
-                CK(cudaMemsetAsync(c->s.zq, 0, fma_code_words(c->max_d) * sizeof(uint2), st));
-                c->epoch = 1;
-            }
-            CK(fma_head(hm, A, Bm, mrows, fp.mt, d, r, V, kk, mode, ids_t, lp_t, lg_t, c->s, c->epoch, c->sm_count, st));
+            unsigned int epoch = 0;
+            CK(next_epoch(c, st, &epoch));
+            CK(fma_head(hm, A, Bm, mrows, fp.mt, d, r, V, kk, mode, ids_t, lp_t, lg_t, c->s, epoch, c->sm_count, st));
             nl += 1;
         } else if (use_slab) {
             const bf16* const zp[3] = {lowrank ? c->s.zb : hm, lowrank ? c->s.zb_lo : nullptr, nullptr};

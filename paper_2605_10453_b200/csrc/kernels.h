@@ -17,11 +17,8 @@ struct Scratch {
     bf16* zb;            // bf16 code [M][r] for the tensor-core path
     bf16* zb_lo;         // its rounding remainder (z - zb), bf16: used while the call is HBM-bound
     bf16* zb_lo2;        // what the two leave: up to 64 rows, for the shapes that keep all of fp32
-    float* zpart;        // K-split partial tiles of the tensor-core down-projection
-    size_t zpart_elems;
-    uint32_t* smax;      // tensor path: per-row maxima of the sample tiles [64][M padded to 128]
-    size_t smax_elems;
-    uint32_t* thr0;      // tensor path: per-row starting bound of the top-k lists
+    unsigned long long* bound;   // tensor path: per row up to 32 words (call number, key) that bound its k-th largest logit
+    int bound_pitch;     // rows of it
     float* part;         // split-V partial records
     size_t part_elems;
     unsigned int* tickets;  // arrival counter: it only counts up
@@ -101,18 +98,23 @@ cudaError_t slab_head(const bf16* const (&z)[3], int z_pitch, const bf16* W, int
 cudaError_t merge_records(const float* part, int M, int P, int k, int32_t* ids, float* logprobs, cudaStream_t st);
 
 // ---- tensor-core path (larger M) ------------------------------------------------------
-// Shapes the tcgen05 kernels take: K a multiple of 64, N a multiple of 8 and >= 64, k <= 32 in top-k mode.
-bool tensor_ok(int M, int K, int N, int k, int mode);
-// z (bf16 [M][r], in s.zb) = h A; with_low_part also writes s.zb_lo = bf16(z - zb).
-cudaError_t tensor_downproj(const bf16* h, const bf16* A, int M, int d, int r, bool with_low_part, const Scratch& s,
+// Once per device, before the first launch.
+cudaError_t tensor_prepare();
+// Shapes the tcgen05 kernels take: K of at least 64 (full rank: a multiple of 8), N a multiple of 8 and >= 64, k <= 32 in top-k mode.
+bool tensor_ok(int M, bool lowrank, int K, int N, int k, int mode);
+// ... and their down-projection.
+bool tensor_code_ok(int d, int r);
+// z (bf16 [M][z_pitch]) = h A, and z_lo, if not null, = bf16(h A - z).
+cudaError_t tensor_downproj(const bf16* h, const bf16* A, int M, int d, int r, bf16* z, bf16* z_lo, int z_pitch, const Scratch& s,
                             int sm_count, int* launches, cudaStream_t st);
-// X W with X bf16 [M][K], W bf16 [K][N]; mode 0: fused log-softmax / top-k, mode 1: raw fp32 logits.
-// Xlo, if not null, is added to X inside the contraction (two MMAs per step).
-// ev0 / ev1, if not null, are recorded directly before / after the kernel that streams W.
 // tensor_records_fit: does the context's record scratch take this call?
 bool tensor_records_fit(int M, int N, int k, const Scratch& s, int sm_count);
-cudaError_t tensor_head(const bf16* X, const bf16* Xlo, const bf16* W, int M, int K, int N, int k, int mode, int32_t* ids,
-                        float* logprobs, float* logits, const Scratch& s, int sm_count, int* launches,
+// X W with X bf16 [M][K], rows x_pitch elements apart, W bf16 [K][N]; mode 0: fused log-softmax / top-k, mode 1: raw fp32 logits.
+// Xlo, if not null, is added to X inside the contraction (two MMAs per step).  epoch: larger than every earlier
+// call's on this scratch and never 0.
+// ev0 / ev1, if not null, are recorded directly before / after the kernel that streams W.
+cudaError_t tensor_head(const bf16* X, const bf16* Xlo, int x_pitch, const bf16* W, int M, int K, int N, int k, int mode, int32_t* ids,
+                        float* logprobs, float* logits, const Scratch& s, unsigned int epoch, int sm_count, int* launches,
                         cudaEvent_t ev0, cudaEvent_t ev1, cudaStream_t st);
 
 }  // namespace slimspec

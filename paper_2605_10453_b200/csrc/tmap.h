@@ -44,22 +44,38 @@ inline bool make_map(CUtensorMap* map, const void* base, int rows, int cols, int
 }
 
 // Launch with (or without) the programmatic-dependent-launch attribute: the kernel may start while
-// the one before it in the stream is still running and meets it at griddepcontrol.wait.
+// the one before it in the stream is still running and meets it at griddepcontrol.wait.  cluster: CTAs of a cluster.
 template <typename... KArgs, typename... Args>
-static cudaError_t launch_chain(void (*kern)(KArgs...), int grid, int block, size_t smem, bool pdl, cudaStream_t st,
-                                Args... args)
+static cudaError_t launch_chain_cluster(void (*kern)(KArgs...), int grid, int cluster, int block, size_t smem, bool pdl, cudaStream_t st,
+                                        Args... args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(grid);
     cfg.blockDim = dim3(block);
     cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
+    int n = 0;
+    if (pdl) {
+        attr[n].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[n++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        attr[n].id = cudaLaunchAttributeClusterDimension;
+        attr[n].val.clusterDim.x = (unsigned)cluster;
+        attr[n].val.clusterDim.y = 1;
+        attr[n++].val.clusterDim.z = 1;
+    }
     cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
+    cfg.numAttrs = n;
     return cudaLaunchKernelEx(&cfg, kern, args...);
+}
+
+template <typename... KArgs, typename... Args>
+static cudaError_t launch_chain(void (*kern)(KArgs...), int grid, int block, size_t smem, bool pdl, cudaStream_t st,
+                                Args... args)
+{
+    return launch_chain_cluster(kern, grid, 1, block, smem, pdl, st, args...);
 }
 
 }  // namespace slimspec
