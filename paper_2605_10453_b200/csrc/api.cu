@@ -40,7 +40,15 @@ static const int kSplitCodeRows = 256;  // tensor path: z carried as hi + lo bf1
 static const int kRowPad = 8;          // rows of the generic path's fp32 code are padded to this
 static const int kStreamTile = 16;     // rows one launch of the older streaming kernels takes
 static const int kSlabRows = 64;       // rows one launch of the slab kernel takes
-static const int kCodeByStreamRows = 32;   // tensor path: up to this many rows z comes from the streaming path's down-projection
+
+// Which down-projection.  The streaming path's (small CTAs that come up beside the kernel before) reads A once per 16 rows; the
+// tensor cores' reads it once, with about 5 us more of its own.  Measured, whole call, streaming / tensor: 16 rows d = 4096,
+// r = 512: 38.1 / 42.3 us, r = 1024 (V = 64000): 40.5 / 44.7, d = 8192, r = 1024: 74.3 / 64.1; 32 rows d = 4096,
+// r = 512: 41.8 / 47.5, d = 5120, r = 640: 67.8 / 62.7, d = 8192, r = 2048: 142.9 / 113.3; 64 rows d = 8192, r = 1024: 115 / 82.
+static bool code_by_tensor(int M, int d, int r) { return tensor_code_ok(d, r) && (M > 32 || (long long)d * r * ((M + 15) / 16) > (4ll << 20)); }
+// From how many elements of the contraction on 33 to 64 rows run on the tensor path rather than on the slab kernel (64 rows,
+// slab / tensor: r = 128 36.1 / 40.3 us, 512 60.2 / 49.7, 1024 86.4 / 73.5, 2048 140 / 124, full rank 4096 179 / 174).
+static const int kTensorManyK = 320;
 
 static int round_up(int x, int m) { return (x + m - 1) / m * m; }
 
@@ -273,7 +281,7 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
     const bool tensor_fits = tensor_ok(M, lowrank, K, V, k, mode) && ptr_ok;
     if (path == SLIMSPEC_PATH_AUTO) {
         // FP32 FMAs keep up with HBM only for a few rows; beyond that the tensor cores take over
-        if (M > (slab ? kSlabRows : kStreamMaxRows) && tensor_fits) path = SLIMSPEC_PATH_TENSOR;
+        if (M > (slab ? (K >= kTensorManyK ? 32 : kSlabRows) : kStreamMaxRows) && tensor_fits) path = SLIMSPEC_PATH_TENSOR;
         else path = stream_ok ? SLIMSPEC_PATH_STREAM : (tensor_fits ? SLIMSPEC_PATH_TENSOR : SLIMSPEC_PATH_GENERIC);
     }
     if (path == SLIMSPEC_PATH_TENSOR && !tensor_fits) return SLIMSPEC_ERR_ALIGN;
@@ -340,7 +348,7 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
             // remainder of z and feed it through a second MMA, so z is effectively fp32-exact.
             const bool low_part = M <= kSplitCodeRows;
             cudaError_t e0;
-            if (M > kCodeByStreamRows && tensor_code_ok(d, r)) {
+            if (code_by_tensor(M, d, r)) {
                 e0 = tensor_downproj(h, A, M, d, r, c->s.zb, low_part ? c->s.zb_lo : nullptr, x_pitch, c->s, c->sm_count, &n, st);
             } else {
                 // few rows: the streaming path's down-projection (one launch of small CTAs) is the faster one; it also takes every shape
@@ -381,9 +389,7 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
         const bool fma = fp.ok && fp.ncta <= c->s.max_parts;
         const bool use_slab = !fma && slab && slab_ok(mrows, lowrank, K, V, kk, c->sm_count);
         if (use_slab) {
-            // the streaming path's down-projection reads A once per 16 rows: beyond 32 the K-split tensor-core product
-            // and its reduction are faster (64 rows, d = 8192, r = 1024: whole call 115.5 us with the one, 81.7 us with the other)
-            if (lowrank && mrows > kCodeByStreamRows && tensor_code_ok(d, r)) CK(tensor_downproj(hm, A, mrows, d, r, c->s.zb, c->s.zb_lo, r, c->s, c->sm_count, &nl, st));
+            if (lowrank && code_by_tensor(mrows, d, r)) CK(tensor_downproj(hm, A, mrows, d, r, c->s.zb, c->s.zb_lo, r, c->s, c->sm_count, &nl, st));
             else if (lowrank) {
                 bf16* const zp[3] = {c->s.zb, c->s.zb_lo, nullptr};
                 CK(stream_code_rows(hm, A, mrows, d, r, r, zp, c->sm_count, st));

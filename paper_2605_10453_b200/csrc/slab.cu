@@ -331,7 +331,9 @@ __global__ void __maxnreg__(RAGGED ? 96 : 112) k_slab_head(const __grid_constant
         }
         __syncwarp();
     } else if (warp == 1) {
-        // ================= MMA issuer: per stage two steps of 16 along K for every tile
+        // ================= MMA issuer: per stage two steps of 16 along K for every tile.  All tiles get one part of the code
+        // before any gets the next: two instructions in a row into the same accumulator wait for one another (64 rows,
+        // d = 8192, r = 1024: 115 us part by part in each tile, 86 us this way).
         if (lane == 0) {
             constexpr uint32_t A_HI = (1024u >> 4) | (1u << 14) | (2u << 29);      // SBO: 8 rows of K; version 1; 128-byte swizzle
             constexpr uint32_t B_HI = (512u >> 4) | (1u << 14) | (4u << 29);       // SBO: 8 rows of z; 64-byte swizzle
@@ -347,14 +349,15 @@ __global__ void __maxnreg__(RAGGED ? 96 : 112) k_slab_head(const __grid_constant
                 const uint32_t st = ring_w + (uint32_t)s * stage_w;
 #pragma unroll
                 for (int kk = 0; kk < 2; ++kk) {
-                    uint32_t a = (st + (uint32_t)(kk * 128)) | a_lbo, d = tmem_base;
-                    const uint32_t b = (st + z_off + (uint32_t)(kk * 2)) | (1u << 16);
-                    const uint32_t acc = (i | kk) ? 1u : 0u;
-                    for (int t = 0; t < ntile; ++t) {
-                        tc_mma_bf16_words2(d, a, A_HI, b, B_HI, p.idesc, acc);
-                        for (int q = 1; q <= more; ++q) tc_mma_bf16_words2(d, a, A_HI, b + (uint32_t)q * z_part, B_HI, p.idesc, 1u);
-                        a += (uint32_t)(2 * kSlabBox) >> 4;
-                        d += (uint32_t)p.tcols;
+                    for (int q = 0; q <= more; ++q) {
+                        uint32_t a = (st + (uint32_t)(kk * 128)) | a_lbo, d = tmem_base;
+                        const uint32_t b = (st + z_off + (uint32_t)(kk * 2) + (uint32_t)q * z_part) | (1u << 16);
+                        const uint32_t acc = (i | kk | q) ? 1u : 0u;
+                        for (int t = 0; t < ntile; ++t) {
+                            tc_mma_bf16_words2(d, a, A_HI, b, B_HI, p.idesc, acc);
+                            a += (uint32_t)(2 * kSlabBox) >> 4;
+                            d += (uint32_t)p.tcols;
+                        }
                     }
                 }
                 tc_commit(&empty[s]);

@@ -70,3 +70,21 @@ def test_batch_equal_logits(ctx, M):
     assert ctx.last_error() == binding.OK and ctx.last_path() == binding.PATH_TENSOR
     assert check_topk(oracle.fullhead_topk(oracle.bf16_bits(h), oracle.bf16_bits(W.cpu()), k), ids.cpu().numpy(), lp.cpu().numpy())["max_lp_err"] < 1e-4
     assert ids[M // 2:].cpu().tolist() == [list(range(k))] * (M - M // 2)
+
+
+@pytest.mark.parametrize("M,d,r,V,k,path", [
+    (33, 512, 328, 8 * 1001, 10, binding.PATH_TENSOR),       # 33 to 64 rows: from a rank of 320 on
+    (64, 1024, 320, 256 * 150, 20, binding.PATH_TENSOR),
+    (17, 4104, 528, 8 * 3000, 10, binding.PATH_STREAM),      # slab kernel behind the tensor cores' down-projection
+    (3, 4104, 1040, 8 * 1777, 5, binding.PATH_STREAM),
+])
+def test_few_rows_matches_oracle(M, d, r, V, k, path):
+    ctx = binding.Context(max_M=M, max_d=d, max_V=V, max_k=k)
+    x = synth.make_inputs(M, d, r, V, seed=37)
+    g = {n: t.to(DEV) for n, t in x.items()}
+    b = {n: oracle.bf16_bits(t) for n, t in x.items()}
+    ids, lp = ctx.slimspec_head_topk(g["h"], g["A"], g["B"], k)
+    torch.cuda.synchronize()
+    assert ctx.last_error() == binding.OK and ctx.last_path() == path
+    ctx.close()
+    assert check_topk(oracle.head_topk(b["h"], b["A"], b["B"], k), ids.cpu().numpy(), lp.cpu().numpy())["max_lp_err"] < 1e-4
