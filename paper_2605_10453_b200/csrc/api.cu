@@ -122,7 +122,7 @@ extern "C" int slimspec_create(slimspec_ctx** out, int max_M, int max_d, int max
     ok = ok && cudaMemset(c->s.zq, 0, fma_code_words(max_d) * sizeof(uint2)) == cudaSuccess;
     ok = ok && cudaMemset(c->s.z, 0, z_elems * sizeof(float)) == cudaSuccess;
     ok = ok && cudaMemset(c->s.bound, 0, 32 * mpad128 * sizeof(unsigned long long)) == cudaSuccess;
-    ok = ok && stream_prepare() == cudaSuccess && slab_prepare() == cudaSuccess && tensor_prepare() == cudaSuccess && fma_prepare() == cudaSuccess;
+    ok = ok && stream_prepare() == cudaSuccess && slab_prepare() == cudaSuccess && tensor_prepare(c->s.max_clusters) == cudaSuccess && fma_prepare() == cudaSuccess;
     ok = ok && cudaDeviceSynchronize() == cudaSuccess;
     if (!ok) {
         cudaGetLastError();

@@ -19,6 +19,7 @@ struct Scratch {
     bf16* zb_lo2;        // what the two leave: up to 64 rows, for the shapes that keep all of fp32
     unsigned long long* bound;   // tensor path: per row up to 32 words (call number, key) that bound its k-th largest logit
     int bound_pitch;     // rows of it
+    int max_clusters[9];         // tensor path: clusters of that many CTAs of the down-projection that run at the same time
     float* part;         // split-V partial records
     size_t part_elems;
     unsigned int* tickets;  // arrival counter: it only counts up
@@ -98,8 +99,9 @@ cudaError_t slab_head(const bf16* const (&z)[3], int z_pitch, const bf16* W, int
 cudaError_t merge_records(const float* part, int M, int P, int k, int32_t* ids, float* logprobs, cudaStream_t st);
 
 // ---- tensor-core path (larger M) ------------------------------------------------------
-// Once per device, before the first launch.
-cudaError_t tensor_prepare();
+static constexpr int kTcMaxSplits = 8;       // CTAs that share the K of a tile of the down-projection (a portable cluster)
+// Once per device, before the first launch; says how many clusters of 1 .. kTcMaxSplits CTAs run at the same time.
+cudaError_t tensor_prepare(int (&max_clusters)[kTcMaxSplits + 1]);
 // Shapes the tcgen05 kernels take: K of at least 64 (full rank: a multiple of 8), N a multiple of 8 and >= 64, k <= 32 in top-k mode.
 bool tensor_ok(int M, bool lowrank, int K, int N, int k, int mode);
 // ... and their down-projection.

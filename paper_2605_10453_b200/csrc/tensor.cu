@@ -33,7 +33,7 @@ static constexpr int kTcEpiThreads = kTcEpiWarps * 32;
 // shared memory the final sort of the lists needs (values and ids of every epilogue thread)
 static constexpr size_t kTcSortBytes = (size_t)kTcEpiThreads * kTcListPitch * 8;
 static constexpr int kTcMaxStages = 8;
-static constexpr int kTcMaxSplits = 8;       // CTAs that share the K of a tile of the down-projection (a portable cluster)
+static constexpr int kTcMaxResident = 16;    // most K chunks of a resident X
 static constexpr int kTcPartPitch = 132;     // floats between two rows of a partial tile in shared memory: 33 16-byte units, odd
 static constexpr int kTcBoundPolls = 32;     // looks at the other CTAs' maxima after the first tile
 static constexpr float kLog2e = 1.4426950408889634f;
@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
                                ((uint32_t)(NV >> 3) << 17) | ((uint32_t)((CG * kTcRows) >> 4) << 24);
 
     extern __shared__ unsigned char smem_raw[];
-    __shared__ uint64_t full[kTcMaxStages], empty[kTcMaxStages], acc_full[2], acc_empty[2], x_full;
+    __shared__ uint64_t full[kTcMaxStages], empty[kTcMaxStages], acc_full[2], acc_empty[2], x_full[kTcMaxResident];
     __shared__ uint32_t tmem_base_s;
     __shared__ int abort_s;
     unsigned char* xarea = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
@@ -225,7 +225,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
     if (tid == 0) {
         for (int s = 0; s < NS; ++s) { mbar_init(&full[s], 1); mbar_init(&empty[s], 1); }
         for (int b = 0; b < 2; ++b) { mbar_init(&acc_full[b], 1); mbar_init(&acc_empty[b], CG * kTcEpiWarps); }
-        mbar_init(&x_full, 1);
+        for (int c = 0; c < kTcMaxResident; ++c) mbar_init(&x_full[c], 1);
         abort_s = 0;
         mbar_fence_init();
         prefetch_tensor_map(&p.mapX);
@@ -251,7 +251,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
         if (lane == 0) {
             // Barriers of a pair are the first CTA's: it expects the bytes of both.
             const uint32_t full0 = CG == 2 ? cluster_map(smem_u32(&full[0]), 0) : smem_u32(&full[0]);
-            const uint32_t xfull0 = CG == 2 ? cluster_map(smem_u32(&x_full), 0) : smem_u32(&x_full);
+            const uint32_t xfull0 = CG == 2 ? cluster_map(smem_u32(&x_full[0]), 0) : smem_u32(&x_full[0]);
             const bool first_cta = CG == 1 || rank == 0;
             auto load = [&](unsigned char* dst, const CUtensorMap* map, int x, int y, uint32_t bar0, uint64_t* bar_here) {
                 if (CG == 2) tma_load_2d_pair(dst, map, x, y, bar0);
@@ -272,8 +272,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
             for (int i = 0; i < npre; ++i) send_w(i, cg + (i / cps) * p.gct, i % cps);
             pdl_wait();
             if (xres && ntiles > 0) {
-                if (first_cta) mbar_arrive_expect_tx(&x_full, (uint32_t)(CG * cps * XB));
-                for (int c = 0; c < cps; ++c) send_x(xarea + (size_t)c * XB, c, xfull0, &x_full);
+                for (int c = 0; c < cps; ++c) {
+                    if (first_cta) mbar_arrive_expect_tx(&x_full[c], (uint32_t)(CG * XB));
+                    send_x(xarea + (size_t)c * XB, c, xfull0 + (uint32_t)(c * 8), &x_full[c]);
+                }
             }
             // ring positions are kept as (slot, phase) pairs: no division on this thread's path
             int s = 0, ph = 0, i = 0;
@@ -306,7 +308,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
             int s = 0, ph = 0;
             uint32_t st = ring_w;
             bool alive = true;
-            if (xres && ntiles > 0 && !mbar_wait(&x_full, 0, abort_flag, p.err, ERR_WAIT_FULL)) alive = false;
             for (int t = 0; t < ntiles && alive; ++t) {
                 const int buf = t & 1;
                 if (t >= 2 && !mbar_wait(&acc_empty[buf], ((t >> 1) - 1) & 1, abort_flag, p.err, ERR_WAIT_FREE)) break;
@@ -314,6 +315,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * NV);
                 uint32_t xr = xres_w;
                 for (int c = 0; c < cps; ++c) {
+                    if (t == 0 && xres && !mbar_wait(&x_full[c], 0, abort_flag, p.err, ERR_WAIT_FULL)) { alive = false; break; }
                     if (!mbar_try_wait(&full[s], ph) && !mbar_wait(&full[s], ph, abort_flag, p.err, ERR_WAIT_FULL)) { alive = false; break; }
                     const uint32_t a_lo = xres ? xr : st | (1u << 16);
                     const uint32_t b_lo = (st + (xres ? 0u : a_step)) | ((uint32_t)(WBOX_BYTES >> 4) << 16);
@@ -352,7 +354,6 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
         const int m = rb * kTcRows + row;
         const bool live = m < p.M, warp_live = rb * kTcRows + quarter * 32 < p.M;
         const int k = p.k;
-        constexpr int NCH = NV / 2 / 32;          // chunks of 32 columns per warp and tile: 2 or 4
         const uint32_t acc_empty0 = CG == 2 ? cluster_map(smem_u32(&acc_empty[0]), 0) : smem_u32(&acc_empty[0]);
         EpiRow st;
         st.run_max = -FLT_MAX;
@@ -369,15 +370,25 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
             if (!mbar_wait_warp(&acc_full[buf], (t >> 1) & 1, abort_flag, p.err, ERR_WAIT_ACC)) { alive = false; break; }
             tc_fence_after_sync();
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * NV + half * (NV / 2));
-            if (p.mode == 0 && warp_live) {
+            // The warp has read what it needs of the buffer.
+            auto hand_back = [&] {
+                tc_fence_before_sync();
+                __syncwarp();
+                if (lane == 0) {
+                    if (CG == 2) mbar_arrive_cluster(acc_empty0 + (uint32_t)(buf * 8));
+                    else mbar_arrive(&acc_empty[buf]);
+                }
+            };
+            const int ncol = warp_live ? min(NV / 2, p.N - colbase) : 0;      // the warp's columns of this tile; may be negative
+            if (p.mode == 0 && ncol > 0) {
 #pragma unroll 1
-                for (int i = 0; i < NCH; ++i) {
-                    const int nvalid = p.N - (colbase + i * 32);      // same for every thread
-                    if (nvalid <= 0) break;
+                for (int i = 0; i < ncol; i += 32) {
                     uint32_t v[32];
-                    tmem_ld_32x32(taddr + (uint32_t)(i * 32), v);
+                    tmem_ld_32x32(taddr + (uint32_t)i, v);
                     tmem_ld_wait();
-                    epi_chunk(v, nvalid, colbase + i * 32, k, t > 0, st, list);
+                    // the next MMAs into this buffer start while the last columns are worked on
+                    if (i + 32 >= ncol && t > 0) hand_back();
+                    epi_chunk(v, ncol - i, colbase + i, k, t > 0, st, list);
                 }
                 if (((t + 1) & t) == 0 && live) bound_publish(p, group, m, st.run_max);
                 if (t == 0) {
@@ -389,9 +400,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
                     } while (++polls < kTcBoundPolls && 2 * p.gct >= k && __any_sync(0xffffffffu, live && b == -FLT_MAX));
                     st.thr = fmaxf(st.thr, b);
                     // with the bound, the first tile once more, for its candidates
-                    const int ng = min(NV / 2, p.N - colbase) / 8;
 #pragma unroll 1
-                    for (int g = 0; g < ng; ++g) {
+                    for (int g = 0; g < ncol / 8; ++g) {
                         uint32_t w[8];
                         tmem_ld(taddr + (uint32_t)(g * 8), w);
                         tmem_ld_wait();
@@ -401,56 +411,61 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
                         epi_park(x, colbase + g * 8, k, st, list);
                         __syncwarp();
                     }
+                    hand_back();
                 }
-            } else if (p.mode == 1 && warp_live) {
+                continue;
+            }
+            if (p.mode == 1) {
                 float* dst = p.out + (size_t)m * p.N + colbase;
 #pragma unroll 1
-                for (int i = 0; i < NCH; ++i) {
-                    const int nvalid = p.N - (colbase + i * 32);
-                    if (nvalid <= 0) break;
+                for (int i = 0; i < ncol; i += 32) {
                     uint32_t v[32];
-                    tmem_ld_32x32(taddr + (uint32_t)(i * 32), v);
+                    tmem_ld_32x32(taddr + (uint32_t)i, v);
                     tmem_ld_wait();
 #pragma unroll
                     for (int e = 0; e < 32; e += 4) {
-                        if (live && e < nvalid)      // N is a multiple of 8, so a group of four is all in or all out
-                            *reinterpret_cast<float4*>(dst + i * 32 + e) = make_float4(__uint_as_float(v[e]), __uint_as_float(v[e + 1]), __uint_as_float(v[e + 2]), __uint_as_float(v[e + 3]));
+                        if (live && i + e < ncol)      // N is a multiple of 8, so a group of four is all in or all out
+                            *reinterpret_cast<float4*>(dst + i + e) = make_float4(__uint_as_float(v[e]), __uint_as_float(v[e + 1]), __uint_as_float(v[e + 2]), __uint_as_float(v[e + 3]));
                     }
                 }
-            } else if (p.mode == 2 && warp_live) {
+            } else if (p.mode == 2) {
                 // the partial tile, to shared memory: every MMA has completed, the ring is idle
                 float* dst = reinterpret_cast<float*>(xarea) + (size_t)row * kTcPartPitch + half * (NV / 2);
 #pragma unroll 1
-                for (int i = 0; i < NCH; ++i) {
+                for (int i = 0; i < ncol; i += 32) {
                     uint32_t v[32];
-                    tmem_ld_32x32(taddr + (uint32_t)(i * 32), v);
+                    tmem_ld_32x32(taddr + (uint32_t)i, v);
                     tmem_ld_wait();
 #pragma unroll
                     for (int e = 0; e < 32; e += 4)
-                        *reinterpret_cast<float4*>(dst + i * 32 + e) = make_float4(__uint_as_float(v[e]), __uint_as_float(v[e + 1]), __uint_as_float(v[e + 2]), __uint_as_float(v[e + 3]));
+                        *reinterpret_cast<float4*>(dst + i + e) = make_float4(__uint_as_float(v[e]), __uint_as_float(v[e + 1]), __uint_as_float(v[e + 2]), __uint_as_float(v[e + 3]));
                 }
             }
-            tc_fence_before_sync();
-            __syncwarp();
-            if (lane == 0) {
-                if (CG == 2) mbar_arrive_cluster(acc_empty0 + (uint32_t)(buf * 8));
-                else mbar_arrive(&acc_empty[buf]);
-            }
+            hand_back();
         }
         if (alive && live && p.mode == 0 && ntiles > 0) {
-            // The lists live in local memory, which this kernel's small L1 hardly caches: a sort
-            // there pays an L2 round trip per step.  Every MMA has completed by now (the last
-            // accumulator was handed over), so the operand rings are dead: sort in that memory.
+            // The lists live in local memory, which this kernel's small L1 hardly caches.  Every MMA has completed by
+            // now (the last accumulator was handed over), so the operand rings are dead: the list is put in order there, an
+            // entry's place being the number of better ones (of equal values the earlier has the lower id).
             uint2* sl = reinterpret_cast<uint2*>(xarea) + (size_t)(warp * 32 + lane) * kTcListPitch;
-            int cnt = st.cnt;
+            const int cnt = st.cnt;
             for (int j = 0; j < cnt; ++j) sl[j] = list[j];
-            topk_compact(sl, cnt, k, st.thr);
-            const int P = 2 * p.gct;
-            *rec_pair(p.part, m, P, k, 2 * cg + half, 0) = make_float2(st.run_max, st.run_sum);
-            // (key, id) pairs; -0 and +0 rank alike.  The merge looks at the first three and then on to the first empty one.
+            const int P = 2 * p.gct, slab = 2 * cg + half;
+            *rec_pair(p.part, m, P, k, slab, 0) = make_float2(st.run_max, st.run_sum);
+            for (int j = 0; j < cnt; ++j) {
+                const uint2 mine = sl[j];
+                int rank = 0;
+#pragma unroll 4
+                for (int i = 0; i < cnt; ++i) {
+                    const float o = __uint_as_float(sl[i].x);
+                    rank += o > __uint_as_float(mine.x) || (o == __uint_as_float(mine.x) && i < j) ? 1 : 0;
+                }
+                // (key, id) pairs; -0 and +0 rank alike
+                if (rank < k) *rec_pair(p.part, m, P, k, slab, 1 + rank) = make_float2(__uint_as_float(f2key(__uint_as_float(mine.x) + 0.f)), __int_as_float((int)mine.y));
+            }
+            // the merge looks at the first three and then on to the first empty one
             const int nw = min(k, max(cnt + 1, 3));
-            for (int j = 0; j < nw; ++j)
-                *rec_pair(p.part, m, P, k, 2 * cg + half, 1 + j) = make_float2(__uint_as_float(j < cnt ? f2key(__uint_as_float(sl[j].x) + 0.f) : 0u), __int_as_float(j < cnt ? (int)sl[j].y : kNoId));
+            for (int j = cnt; j < nw; ++j) *rec_pair(p.part, m, P, k, slab, 1 + j) = make_float2(__uint_as_float(0u), __int_as_float(kNoId));
         }
     }
     // ---- teardown: every role is past its last use of tensor memory
@@ -544,7 +559,7 @@ static cudaError_t launch_gemm(TcParams p, int grid, bool pdl, cudaStream_t st)
 {
     const size_t x_bytes = (size_t)p.xbox_bytes * (p.split ? 2 : 1), w_bytes = (size_t)kTcKChunk * (NV / CG) * 2;
     const size_t x_all = (size_t)((p.chunks + p.nks - 1) / p.nks) * x_bytes;
-    p.xres = (p.mode != 2 && x_all + 4 * w_bytes + 1024 <= kTcSmemMax) ? 1 : 0;
+    p.xres = (p.mode != 2 && p.chunks <= kTcMaxResident && x_all + 4 * w_bytes + 1024 <= kTcSmemMax) ? 1 : 0;
     const size_t fixed = 1024 + (p.xres ? x_all : 0);
     const size_t stage = w_bytes + (p.xres ? 0 : x_bytes);
     int ns = (int)((kTcSmemMax - fixed) / stage);
@@ -558,12 +573,27 @@ static cudaError_t launch_gemm(TcParams p, int grid, bool pdl, cudaStream_t st)
     return launch_chain_cluster(k_tc_gemm<CG, NV>, grid, CG == 2 ? 2 : p.nks, kTcThreads, smem, pdl, st, p);
 }
 
-cudaError_t tensor_prepare()
+cudaError_t tensor_prepare(int (&max_clusters)[kTcMaxSplits + 1])
 {
     cudaError_t e;
     if ((e = cudaFuncSetAttribute(k_tc_gemm<1, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemMax)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_tc_gemm<1, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemMax)) != cudaSuccess) return e;
-    return cudaFuncSetAttribute(k_tc_gemm<2, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemMax);
+    if ((e = cudaFuncSetAttribute(k_tc_gemm<2, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemMax)) != cudaSuccess) return e;
+    max_clusters[0] = max_clusters[1] = 1 << 30;
+    for (int c = 2; c <= kTcMaxSplits; ++c) {
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = dim3(c);
+        cfg.blockDim = dim3(kTcThreads);
+        cfg.dynamicSmemBytes = kTcSmemMax;
+        cudaLaunchAttribute attr;
+        attr.id = cudaLaunchAttributeClusterDimension;
+        attr.val.clusterDim.x = (unsigned)c;
+        attr.val.clusterDim.y = attr.val.clusterDim.z = 1;
+        cfg.attrs = &attr;
+        cfg.numAttrs = 1;
+        if ((e = cudaOccupancyMaxActiveClusters(&max_clusters[c], k_tc_gemm<1, 128>, &cfg)) != cudaSuccess) return e;
+    }
+    return cudaSuccess;
 }
 
 struct TcShape {
@@ -652,10 +682,10 @@ cudaError_t tensor_downproj(const bf16* h, const bf16* A, int M, int d, int r, b
     p.nrb = (M + kTcRows - 1) / kTcRows;
     p.nct = (r + 127) / 128;
     p.chunks = (d + kTcKChunk - 1) / kTcKChunk;
-    // As many K splits as one wave of clusters takes: of eight CTAs with this much shared memory 15 fit on the chip, of four 33, of two 74 (one
-    // per SM).  (512 rows, d = 4096, r = 512, 16 tiles: 22.6 us with eight splits, two waves; 12 us with four.)
-    int nks = kTcMaxSplits;
-    while (nks > 1 && (nks > p.chunks || nks * p.nrb * p.nct > sm_count - (nks == 8 ? 28 : nks == 4 ? 16 : 0))) nks /= 2;
+    // As many K splits as one wave of clusters takes (fewer clusters fit than SMs suggest: 15 of eight CTAs with this much
+    // shared memory, 33 of four; 512 rows, d = 4096, r = 512, 16 tiles: 22.6 us with eight splits, two waves, 12 us with four).
+    int nks = p.chunks < kTcMaxSplits ? p.chunks : kTcMaxSplits;
+    while (nks > 1 && p.nrb * p.nct > s.max_clusters[nks]) --nks;
     p.nks = nks;
     p.gct = p.nct;
     p.mode = 2;
