@@ -366,7 +366,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
         for (int t = 0; t < ntiles && alive; ++t) {
             const int buf = t & 1;
             const int colbase = (cg + t * p.gct) * NV + half * (NV / 2);
-            if (p.mode == 0 && live && t >= 2 && (t & (t - 1)) == 0) st.thr = fmaxf(st.thr, bound_read(p.bound, p.bound_pitch, p.epoch, k, m));
+            if (p.mode == 0 && live && t >= 1 && (t & (t - 1)) == 0) st.thr = fmaxf(st.thr, bound_read(p.bound, p.bound_pitch, p.epoch, k, m));
             if (!mbar_wait_warp(&acc_full[buf], (t >> 1) & 1, abort_flag, p.err, ERR_WAIT_ACC)) { alive = false; break; }
             tc_fence_after_sync();
             const uint32_t taddr = tmem_base + ((uint32_t)(quarter * 32) << 16) + (uint32_t)(buf * NV + half * (NV / 2));
@@ -382,13 +382,16 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
             const int ncol = warp_live ? min(NV / 2, p.N - colbase) : 0;      // the warp's columns of this tile; may be negative
             if (p.mode == 0 && ncol > 0) {
 #pragma unroll 1
-                for (int i = 0; i < ncol; i += 32) {
-                    uint32_t v[32];
+                for (int i = 0; i < ncol; i += 64) {
+                    uint32_t v[32], w[32];
                     tmem_ld_32x32(taddr + (uint32_t)i, v);
+                    tmem_ld_32x32(taddr + (uint32_t)i + 32, w);
                     tmem_ld_wait();
-                    // the next MMAs into this buffer start while the last columns are worked on
-                    if (i + 32 >= ncol && t > 0) hand_back();
+                    // The next MMAs into this buffer start while the last columns are worked on (handed back before the last 64
+                    // of them rather than 32: 512 rows 86.3 -> 83.2 us, 128 rows 54.8 -> 51.4).
+                    if (i + 64 >= ncol && t > 0) hand_back();
                     epi_chunk(v, ncol - i, colbase + i, k, t > 0, st, list);
+                    if (i + 32 < ncol) epi_chunk(w, ncol - i - 32, colbase + i + 32, k, t > 0, st, list);
                 }
                 if (((t + 1) & t) == 0 && live) bound_publish(p, group, m, st.run_max);
                 if (t == 0) {
