@@ -10,7 +10,7 @@
 // 1.8 KB of consecutive bytes per row at a time.  A bare ring of that shape read 7.1 TB/s here, rings that walk
 // one 128-column tile after another through all of K 6.0 to 6.2 TB/s, the same ring with slabs that do not
 // start on a 128-byte line 5.8 TB/s, boxes of 16 rows 6.0 TB/s (bound by the issue of the TMA
-// instructions, about 50 ns each), four stages in flight 6.8 TB/s against 7.1 TB/s with two.
+// instructions, about 50 ns each as one lane issued them then), four stages in flight 6.8 TB/s against 7.1 TB/s with two.
 // So all tiles of the slab keep their accumulators in tensor memory until the stream has ended: 7 tiles x 64
 // columns for 64 rows and a 128K vocabulary.  z travels with the stages (each 32-column piece is used once).
 // The tensor pipe is idle most of the time: a 128 x N x 16 instruction takes about 32 cycles up to N = 64
@@ -275,7 +275,7 @@ __global__ void __maxnreg__(RAGGED ? 96 : 112) k_slab_head(const __grid_constant
     unsigned char* ring = reinterpret_cast<unsigned char*>(((uintptr_t)smem_raw + 1023) & ~(uintptr_t)1023);
     volatile int* abort_flag = &abort_s;
 
-    const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+    const int tid = threadIdx.x, warp = __shfl_sync(0xffffffffu, tid >> 5, 0), lane = tid & 31;      // the same in all lanes, for the compiler too
     const int cta = blockIdx.x;
     const int my_units = p.units_base + (cta < p.units_rem ? 1 : 0);
     const int col0 = (cta * p.units_base + min(cta, p.units_rem)) * p.unit_cols;
@@ -295,77 +295,90 @@ __global__ void __maxnreg__(RAGGED ? 96 : 112) k_slab_head(const __grid_constant
     tc_fence_before_sync();
     __syncthreads();
     tc_fence_after_sync();
-    const uint32_t tmem_base = tmem_base_s;
+    const uint32_t tmem_base = __shfl_sync(0xffffffffu, tmem_base_s, 0);
 
     if (warp == 0) {
         // ================= producer.  The weights are final before the call is made (the contract of the
         // library), so the first stages' weights are sent for before the kernel ahead has finished; the
         // code comes from that kernel.
-        if (lane == 0) {
-            const uint32_t zpart = (uint32_t)p.zrows * 64u;
-            const uint32_t bytes = (RAGGED ? 0u : (uint32_t)nbox * kSlabBox) + zpart * (uint32_t)p.parts;
-            const int npre = min(p.ns, p.nst);
-            auto send_w = [&](int i, int s) {
-                unsigned char* dst = ring + (size_t)s * p.stage_bytes;
-                mbar_arrive_expect_tx(&full[s], bytes);
-                if (!RAGGED)
-                    for (int b = 0; b < nbox; ++b) tma_load_2d(dst + b * kSlabBox, &p.mapW, col0 + b * 64, i * kSlabStageK, &full[s]);
-            };
-            auto send_z = [&](int i, int s) {
-                unsigned char* dst = ring + (size_t)s * p.stage_bytes + p.wstage_bytes;
-                tma_load_2d(dst, &p.mapZ, i * kSlabStageK, 0, &full[s]);
-                if (p.parts >= 2) tma_load_2d(dst + zpart, &p.mapZ2, i * kSlabStageK, 0, &full[s]);
-                if (p.parts == 3) tma_load_2d(dst + 2 * zpart, &p.mapZ3, i * kSlabStageK, 0, &full[s]);
-            };
+        const uint32_t zpart = (uint32_t)p.zrows * 64u;
+        const uint32_t bytes = (RAGGED ? 0u : (uint32_t)nbox * kSlabBox) + zpart * (uint32_t)p.parts;
+        const int npre = min(p.ns, p.nst);
+        auto send_w = [&](int i, int s) {
+            unsigned char* dst = ring + (size_t)s * p.stage_bytes;
+            mbar_arrive_expect_tx(&full[s], bytes);
+            if (!RAGGED)
+                for (int b = 0; b < nbox; ++b) tma_load_2d(dst + b * kSlabBox, &p.mapW, col0 + b * 64, i * kSlabStageK, &full[s]);
+        };
+        auto send_z = [&](int i, int s) {
+            unsigned char* dst = ring + (size_t)s * p.stage_bytes + p.wstage_bytes;
+            tma_load_2d(dst, &p.mapZ, i * kSlabStageK, 0, &full[s]);
+            if (p.parts >= 2) tma_load_2d(dst + zpart, &p.mapZ2, i * kSlabStageK, 0, &full[s]);
+            if (p.parts == 3) tma_load_2d(dst + 2 * zpart, &p.mapZ3, i * kSlabStageK, 0, &full[s]);
+        };
+        if (elect_one())
             for (int i = 0; i < npre; ++i) send_w(i, i);
-            pdl_launch_dependents();
-            pdl_wait();
-            for (int i = 0; i < npre; ++i) send_z(i, i);
-            int s = 0, ph = 0;
-            for (int i = npre; i < p.nst; ++i) {
-                if (!mbar_wait(&empty[s], ph, abort_flag, p.err, ERR_WAIT_EMPTY)) break;
-                send_w(i, s);
-                send_z(i, s);
-                if (++s == p.ns) { s = 0; ph ^= 1; }
-            }
-        }
         __syncwarp();
+        pdl_launch_dependents();
+        pdl_wait();
+        if (elect_one())
+            for (int i = 0; i < npre; ++i) send_z(i, i);
+        __syncwarp();
+        int s = 0, ph = 0;
+        bool alive = true;
+        for (int i = npre; i < p.nst; ++i) {
+            if (alive) alive = mbar_wait_uniform(&empty[s], ph);
+            if (alive) {
+                if (elect_one()) {
+                    send_w(i, s);
+                    send_z(i, s);
+                }
+                __syncwarp();
+            }
+            if (++s == p.ns) { s = 0; ph ^= 1; }
+        }
+        if (!alive) mbar_gave_up(abort_flag, p.err, ERR_WAIT_EMPTY);
     } else if (warp == 1) {
         // ================= MMA issuer: per stage two steps of 16 along K for every tile.  All tiles get one part of the code
         // before any gets the next: two instructions in a row into the same accumulator wait for one another (64 rows,
         // d = 8192, r = 1024: 115 us part by part in each tile, 86 us this way).
-        if (lane == 0) {
-            constexpr uint32_t A_HI = (1024u >> 4) | (1u << 14) | (2u << 29);      // SBO: 8 rows of K; version 1; 128-byte swizzle
-            constexpr uint32_t B_HI = (512u >> 4) | (1u << 14) | (4u << 29);       // SBO: 8 rows of z; 64-byte swizzle
-            const uint32_t ring_w = (smem_u32(ring) >> 4) & 0x3fffu;
-            const uint32_t a_lbo = (uint32_t)(kSlabBox >> 4) << 16;                // LBO: the tile's second 64 columns
-            const uint32_t stage_w = (uint32_t)p.stage_bytes >> 4, z_off = (uint32_t)p.wstage_bytes >> 4;
-            const uint32_t z_part = (uint32_t)(p.zrows * 64) >> 4;
-            const int more = p.stacked ? 0 : p.parts - 1;
-            int s = 0, ph = 0;
-            bool alive = true;
-            for (int i = 0; i < p.nst; ++i) {
-                if (!mbar_try_wait(&full[s], ph) && !mbar_wait(&full[s], ph, abort_flag, p.err, ERR_WAIT_FULL)) { alive = false; break; }
-                const uint32_t st = ring_w + (uint32_t)s * stage_w;
+        // The warp runs the loop together and elects a lane at each issue (see mbar_wait_uniform).
+        constexpr uint32_t A_HI = (1024u >> 4) | (1u << 14) | (2u << 29);      // SBO: 8 rows of K; version 1; 128-byte swizzle
+        constexpr uint32_t B_HI = (512u >> 4) | (1u << 14) | (4u << 29);       // SBO: 8 rows of z; 64-byte swizzle
+        const uint32_t ring_w = (smem_u32(ring) >> 4) & 0x3fffu;
+        const uint32_t a_lbo = (uint32_t)(kSlabBox >> 4) << 16;                // LBO: the tile's second 64 columns
+        const uint32_t stage_w = (uint32_t)p.stage_bytes >> 4, z_off = (uint32_t)p.wstage_bytes >> 4;
+        const uint32_t z_part = (uint32_t)(p.zrows * 64) >> 4;
+        const int passes = p.stacked ? 1 : p.parts;
+        int s = 0, ph = 0;
+        uint32_t st = ring_w;
+        bool alive = true;
+        for (int i = 0; i < p.nst; ++i) {
+            if (alive) alive = mbar_wait_uniform(&full[s], ph);
+            if (alive) {
+                if (elect_one()) {
 #pragma unroll
-                for (int kk = 0; kk < 2; ++kk) {
-                    for (int q = 0; q <= more; ++q) {
-                        uint32_t a = (st + (uint32_t)(kk * 128)) | a_lbo, d = tmem_base;
-                        const uint32_t b = (st + z_off + (uint32_t)(kk * 2) + (uint32_t)q * z_part) | (1u << 16);
-                        const uint32_t acc = (i | kk | q) ? 1u : 0u;
-                        for (int t = 0; t < ntile; ++t) {
-                            tc_mma_bf16_words2(d, a, A_HI, b, B_HI, p.idesc, acc);
-                            a += (uint32_t)(2 * kSlabBox) >> 4;
-                            d += (uint32_t)p.tcols;
+                    for (int kk = 0; kk < 2; ++kk) {
+                        for (int q = 0; q < passes; ++q) {
+                            uint32_t a = (st + (uint32_t)(kk * 128)) | a_lbo, d = tmem_base;
+                            const uint32_t b = (st + z_off + (uint32_t)(kk * 2) + (uint32_t)q * z_part) | (1u << 16);
+                            const uint32_t acc = (i | kk | q) ? 1u : 0u;
+                            for (int t = 0; t < ntile; ++t) {
+                                tc_mma_bf16_words2(d, a, A_HI, b, B_HI, p.idesc, acc);
+                                a += (uint32_t)(2 * kSlabBox) >> 4;
+                                d += (uint32_t)p.tcols;
+                            }
                         }
                     }
+                    tc_commit(&empty[s]);
+                    if (i == p.nst - 1) tc_commit(&acc_full);
                 }
-                tc_commit(&empty[s]);
-                if (++s == p.ns) { s = 0; ph ^= 1; }
+                __syncwarp();
             }
-            if (alive) tc_commit(&acc_full);
+            st += stage_w;
+            if (++s == p.ns) { s = 0; ph ^= 1; st = ring_w; }
         }
-        __syncwarp();
+        if (!alive) mbar_gave_up(abort_flag, p.err, ERR_WAIT_FULL);
     } else if (RAGGED) {
         // ================= feeders
         SlabFeed f;
