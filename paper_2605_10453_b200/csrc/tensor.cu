@@ -391,7 +391,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
                 }
             };
             const int ncol = warp_live ? min(NV / 2, p.N - colbase) : 0;      // the warp's columns of this tile; may be negative
-            if (p.mode == 0 && ncol > 0) {
+            if (NV >= 128 && p.mode == 0 && ncol > 0) {
 #pragma unroll 1
                 for (int i = 0; i < ncol; i += 64) {
                     uint32_t v[32], w[32];
@@ -437,9 +437,8 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
                     tmem_ld_32x32(taddr + (uint32_t)i, v);
                     tmem_ld_wait();
 #pragma unroll
-                    for (int e = 0; e < 32; e += 4) {
-                        if (live && i + e < ncol)      // N is a multiple of 8, so a group of four is all in or all out
-                            *reinterpret_cast<float4*>(dst + i + e) = make_float4(__uint_as_float(v[e]), __uint_as_float(v[e + 1]), __uint_as_float(v[e + 2]), __uint_as_float(v[e + 3]));
+                    for (int e = 0; e < 32; e += 8) {
+                        if (live && i + e < ncol) st_global_v8(dst + i + e, v + e);      // N is a multiple of 8, so a group of eight is all in or all out
                     }
                 }
             } else if (p.mode == 2) {
@@ -485,14 +484,15 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
     // ---- teardown: every role is past its last use of tensor memory
     tc_fence_before_sync();
     __syncwarp();
-    if (CG == 2 || p.nks > 1) cluster_sync();
+    if (CG == 2) cluster_sync_exec();       // nothing in shared memory is handed over, and the release takes a microsecond
+    else if (p.nks > 1) cluster_sync();
     else __syncthreads();
     tc_fence_after_sync();
     if (warp == kTcMmaWarp) {
         if (CG == 2) tmem_dealloc_pair(tmem_base, 2 * NV);
         else tmem_dealloc(tmem_base, 2 * NV);
     }
-    if (CG == 1 && NV == 128 && p.mode == 2) {
+    if (CG == 1 && NV <= 128 && p.mode == 2) {
         // The code: CTA ks of the cluster adds the partial tiles of its share of the rows, in the order of K, rounds the
         // sum to bf16 and keeps the rounding remainder as a second matrix where the caller wants it.
         const int r0 = ks * kTcRows / p.nks, nr = (ks + 1) * kTcRows / p.nks - r0;
@@ -519,7 +519,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
                 *reinterpret_cast<uint2*>(p.z_lo + (size_t)m * p.z_pitch + col0 + c) = make_uint2(*reinterpret_cast<uint32_t*>(&l01), *reinterpret_cast<uint32_t*>(&l23));
             }
         }
-        if (p.nks > 1) cluster_sync();       // the others have read this CTA's tile
+        if (p.nks > 1) cluster_sync_exec();       // the others have read this CTA's tile
     }
 }
 
@@ -574,13 +574,16 @@ static cudaError_t launch_gemm(TcParams p, int grid, bool pdl, cudaStream_t st)
     const size_t x_bytes = (size_t)p.xbox_bytes * (p.split ? 2 : 1), w_bytes = (size_t)kTcKChunk * (NV / CG) * 2;
     const size_t x_all = (size_t)((p.chunks + p.nks - 1) / p.nks) * x_bytes;
     p.xres = (p.mode != 2 && p.chunks <= kTcMaxResident && x_all + 4 * w_bytes + 1024 <= kTcSmemMax) ? 1 : 0;
-    const size_t fixed = 1024 + (p.xres ? x_all : 0);
     const size_t stage = w_bytes + (p.xres ? 0 : x_bytes);
+    // The MMA reads 128 rows of X, also where a box has fewer; behind the last stage's X there has to be shared memory for that.
+    // (Behind a resident X there is the ring: four stages of 8 KB at least.)
+    const size_t read_to = (size_t)kTcRows * 128 + (p.split ? (size_t)p.xbox_bytes : 0);
+    const size_t over = !p.xres && read_to > stage ? read_to - stage : 0;
+    const size_t fixed = 1024 + (p.xres ? x_all : 0) + over;
     int ns = (int)((kTcSmemMax - fixed) / stage);
     if (ns > kTcMaxStages) ns = kTcMaxStages;
     if (ns < 2) return cudaErrorInvalidValue;
     p.ns = ns;
-    // (The MMA reads 128 rows of X, also where a box has fewer: what follows, 16 KB of weights or more, is still the ring.)
     size_t smem = fixed + (size_t)ns * stage;
     if (p.mode == 0 && smem < 1024 + kTcSortBytes) smem = 1024 + kTcSortBytes;      // room for the final sort of the lists
     if (p.mode == 2 && smem < 1024 + (size_t)kTcRows * kTcPartPitch * 4) smem = 1024 + (size_t)kTcRows * kTcPartPitch * 4;
@@ -593,6 +596,7 @@ cudaError_t tensor_prepare(int (&max_clusters)[kTcMaxSplits + 1])
     if ((e = cudaFuncSetAttribute(k_tc_gemm<1, 128>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemMax)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_tc_gemm<1, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemMax)) != cudaSuccess) return e;
     if ((e = cudaFuncSetAttribute(k_tc_gemm<2, 256>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemMax)) != cudaSuccess) return e;
+    if ((e = cudaFuncSetAttribute(k_tc_gemm<1, 64>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)kTcSmemMax)) != cudaSuccess) return e;
     max_clusters[0] = max_clusters[1] = 1 << 30;
     for (int c = 2; c <= kTcMaxSplits; ++c) {
         cudaLaunchConfig_t cfg = {};
@@ -681,8 +685,8 @@ cudaError_t tensor_head(const bf16* X, const bf16* Xlo, int x_pitch, const bf16*
     return e;
 }
 
-// z = h A through the tensor cores, as bf16 [M][z_pitch] and, if z_lo is not null, its rounding remainder: the K of a 128 x 128
-// tile is split over the CTAs of a cluster, which add their partial tiles through distributed shared memory.
+// z = h A through the tensor cores, as bf16 [M][z_pitch] and, if z_lo is not null, its rounding remainder: the K of a tile of 128
+// rows is split over the CTAs of a cluster, which add their partial tiles through distributed shared memory.
 cudaError_t tensor_downproj(const bf16* h, const bf16* A, int M, int d, int r, bf16* z, bf16* z_lo, int z_pitch, const Scratch& s,
                             int sm_count, int* launches, cudaStream_t st)
 {
@@ -694,7 +698,10 @@ cudaError_t tensor_downproj(const bf16* h, const bf16* A, int M, int d, int r, b
     p.xbox_bytes = xrows * kTcKChunk * 2;
     p.M = M; p.N = r;
     p.nrb = (M + kTcRows - 1) / kTcRows;
-    p.nct = (r + 127) / 128;
+    // Tiles of 64 columns while clusters of four of them fit: half as much to add up per CTA (128 rows, d = 4096, r = 512, whole
+    // call: 51.3 us with tiles of 128 columns, 46.8 with 64; 64 rows 46.0 / 43.3, 512 rows 74.9 / 74.4).
+    const bool narrow = p.nrb * ((r + 63) / 64) <= s.max_clusters[4];
+    p.nct = narrow ? (r + 63) / 64 : (r + 127) / 128;
     p.chunks = (d + kTcKChunk - 1) / kTcKChunk;
     // As many K splits as one wave of clusters takes (fewer clusters fit than SMs suggest: 15 of eight CTAs with this much
     // shared memory, 33 of four; 512 rows, d = 4096, r = 512, 16 tiles: 22.6 us with eight splits, two waves, 12 us with four).
@@ -709,7 +716,7 @@ cudaError_t tensor_downproj(const bf16* h, const bf16* A, int M, int d, int r, b
     // Launched early even as the first kernel of a call: apart from the weights it touches global memory only after its
     // griddepcontrol.wait, so it may come up under the tail of whatever kernel precedes it.
     *launches += 1;
-    return launch_gemm<1, 128>(p, p.nrb * p.nct * nks, true, st);
+    return narrow ? launch_gemm<1, 64>(p, p.nrb * p.nct * nks, true, st) : launch_gemm<1, 128>(p, p.nrb * p.nct * nks, true, st);
 }
 
 }  // namespace slimspec
