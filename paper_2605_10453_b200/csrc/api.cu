@@ -41,11 +41,11 @@ static const int kRowPad = 8;          // rows of the generic path's fp32 code a
 static const int kStreamTile = 16;     // rows one launch of the older streaming kernels takes
 static const int kSlabRows = 64;       // rows one launch of the slab kernel takes
 
-// Which down-projection.  The streaming path's (small CTAs that come up beside the kernel before) reads A once per 16 rows; the
-// tensor cores' reads it once, with about 5 us more of its own.  Measured, whole call, streaming / tensor: 16 rows d = 4096,
-// r = 512: 38.1 / 42.3 us, r = 1024 (V = 64000): 40.5 / 44.7, d = 8192, r = 1024: 74.3 / 64.1; 32 rows d = 4096,
-// r = 512: 41.8 / 47.5, d = 5120, r = 640: 67.8 / 62.7, d = 8192, r = 2048: 142.9 / 113.3; 64 rows d = 8192, r = 1024: 115 / 82.
-static bool code_by_tensor(int M, int d, int r) { return tensor_code_ok(d, r) && (M > 32 || (long long)d * r * ((M + 15) / 16) > (4ll << 20)); }
+// Which down-projection.  The streaming path's (small CTAs that come up beside the kernel before) takes 16 rows at a time and splits d
+// in eight; the tensor cores' takes all rows at once and as many splits as fit.  Measured, whole call, streaming / tensor: 16 rows d = 4096,
+// r = 512: 35.9 / 35.8 us (8 rows 33.4 / 33.9), d = 5120, r = 640: 46.9 / 45.0, d = 8192, r = 512: 45.6 / 37.7; 24 rows d = 2048,
+// r = 512: 26.8 / 26.7, d = 4096, r = 1024: 47.0 / 38.4, d = 5120, r = 640: 59.5 / 50.0; 32 rows d = 8192, r = 2048: 136 / 101.
+static bool code_by_tensor(int M, int d, int r) { return tensor_code_ok(d, r) && (M > 32 || (long long)d * ((M + 15) / 16) > 4096); }
 // From how many elements of the contraction on 33 to 64 rows run on the tensor path rather than on the slab kernel (64 rows,
 // slab / tensor: r = 128 36.1 / 40.3 us, 512 60.2 / 49.7, 1024 86.4 / 73.5, 2048 140 / 124, full rank 4096 179 / 174).
 static const int kTensorManyK = 320;
@@ -275,7 +275,7 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
     const int slab_rows = M < kSlabRows ? M : kSlabRows;
     // (Raw logits of up to 16 rows have no selection to save and stay with the older kernels: M = 4, d = 2048,
     // r = 256: 18.4 us there, 19.4 us here.)
-    const bool slab = ptr_ok && d % 2 == 0 && (!lowrank || r % 16 == 0) && slab_ok(slab_rows, lowrank, K, V, mode == 0 ? k : 1, c->sm_count) &&
+    const bool slab = ptr_ok && d % 2 == 0 && (!lowrank || r % 16 == 0) && slab_ok(slab_rows, lowrank ? 2 : 1, K, V, mode == 0 ? k : 1, c->sm_count) &&
                       !(mode == 1 && M <= kStreamMaxRows && sp.ok);
     const bool stream_ok = (slab && k <= 32) || (sp.ok && ptr_ok && d % 2 == 0 && (!lowrank || r % 16 == 0));
     const bool tensor_fits = tensor_ok(M, lowrank, K, V, k, mode) && ptr_ok;
@@ -347,12 +347,12 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
             // While the call is HBM-bound the tensor cores have time to spare: keep the bf16 rounding
             // remainder of z and feed it through a second MMA, so z is effectively fp32-exact.
             const bool low_part = M <= kSplitCodeRows;
+            bf16* const zp[3] = {c->s.zb, low_part ? c->s.zb_lo : nullptr, nullptr};
             cudaError_t e0;
             if (code_by_tensor(M, d, r)) {
-                e0 = tensor_downproj(h, A, M, d, r, c->s.zb, low_part ? c->s.zb_lo : nullptr, x_pitch, c->s, c->sm_count, &n, st);
+                e0 = tensor_downproj(h, A, M, d, r, zp, x_pitch, c->s, c->sm_count, &n, st);
             } else {
                 // few rows: the streaming path's down-projection (one launch of small CTAs) is the faster one; it also takes every shape
-                bf16* const zp[3] = {c->s.zb, low_part ? c->s.zb_lo : nullptr, nullptr};
                 e0 = stream_code_rows(h, A, M, d, r, x_pitch, zp, c->sm_count, st);
                 n = 1;
             }
@@ -386,12 +386,18 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
         int nl = 0;
         // one or two rows: the FMA kernel, one launch; three to sixteen: the tensor-core streaming kernels
         const FmaPlan fp = fma_plan(mrows, d, lowrank ? r : 0, V, kk, c->sm_count);
-        const bool fma = fp.ok && fp.ncta <= c->s.max_parts;
-        const bool use_slab = !fma && slab && slab_ok(mrows, lowrank, K, V, kk, c->sm_count);
+        // Large A: the slab kernel behind the tensor cores' down-projection, the code in three parts (all of fp32, what the FMA kernel
+        // keeps).  FMA / slab: 4 rows d = 4096, r = 1024, V = 64000 39.7 / 33.4 us, d = 8192, r = 512 40.0 / 35.5, 1024 66.0 / 55.3, 2048 118.7 /
+        // 95.3; 2 rows d = 8192, r = 2048 105.2 / 95.3, but d = 4096, r = 1024 32.5 / 33.3; 1 row r = 2048 100.8 / 95.0, r = 1024 52.6 / 54.9.
+        const bool fma_can = fp.ok && fp.ncta <= c->s.max_parts;
+        const bool slab3 = fma_can && lowrank && slab && slab_ok(mrows, 3, K, V, kk, c->sm_count) && (mrows > 2 || r >= 2048);
+        const bool slab_here = slab3 || (slab && slab_ok(mrows, lowrank ? 2 : 1, K, V, kk, c->sm_count));
+        const bool fma = fma_can && !slab3;
+        const bool use_slab = !fma && slab_here;
         if (use_slab) {
-            if (lowrank && code_by_tensor(mrows, d, r)) CK(tensor_downproj(hm, A, mrows, d, r, c->s.zb, c->s.zb_lo, r, c->s, c->sm_count, &nl, st));
+            bf16* const zp[3] = {c->s.zb, c->s.zb_lo, slab3 ? c->s.zb_lo2 : nullptr};
+            if (lowrank && code_by_tensor(mrows, d, r)) CK(tensor_downproj(hm, A, mrows, d, r, zp, r, c->s, c->sm_count, &nl, st));
             else if (lowrank) {
-                bf16* const zp[3] = {c->s.zb, c->s.zb_lo, nullptr};
                 CK(stream_code_rows(hm, A, mrows, d, r, r, zp, c->sm_count, st));
                 nl = 1;
             }
@@ -416,7 +422,7 @@ static int run_head(slimspec_ctx* c, const bf16* h, const bf16* A, const bf16* B
             CK(fma_head(hm, A, Bm, mrows, fp.mt, d, r, V, kk, mode, ids_t, lp_t, lg_t, c->s, epoch, c->sm_count, st));
             nl += 1;
         } else if (use_slab) {
-            const bf16* const zp[3] = {lowrank ? c->s.zb : hm, lowrank ? c->s.zb_lo : nullptr, nullptr};
+            const bf16* const zp[3] = {lowrank ? c->s.zb : hm, lowrank ? c->s.zb_lo : nullptr, slab3 ? c->s.zb_lo2 : nullptr};
             CK(slab_head(zp, K, Bm, mrows, K, V, kk, mode, ids_t, lp_t, lg_t, c->s, c->sm_count, slot < 0, st));
             nl += 1;
         } else {

@@ -87,7 +87,8 @@ cudaError_t stream_head(const uint32_t* code, bool lowrank, const bf16* B, int M
                         bool after_producer_kernel, int* launches, cudaStream_t st);
 
 // ---- streaming path, up to 64 rows, on the tcgen05 tensor cores (slab.cu) --------------------
-bool slab_ok(int M, bool lowrank, int K, int V, int k, int sm_count);
+// parts: bf16 matrices the code comes in.
+bool slab_ok(int M, int parts, int K, int V, int k, int sm_count);
 // The same for any V, K and alignment of W (the weights then pass through registers).
 bool slab_any_ok(int M, bool lowrank, int K, int V, int k, int sm_count);
 cudaError_t slab_prepare();
@@ -106,8 +107,8 @@ cudaError_t tensor_prepare(int (&max_clusters)[kTcMaxSplits + 1]);
 bool tensor_ok(int M, bool lowrank, int K, int N, int k, int mode);
 // ... and their down-projection.
 bool tensor_code_ok(int d, int r);
-// z (bf16 [M][z_pitch]) = h A, and z_lo, if not null, = bf16(h A - z).
-cudaError_t tensor_downproj(const bf16* h, const bf16* A, int M, int d, int r, bf16* z, bf16* z_lo, int z_pitch, const Scratch& s,
+// h A as bf16 [M][z_pitch] matrices: the value, its rounding remainder, what the two leave (the later ones may be null).
+cudaError_t tensor_downproj(const bf16* h, const bf16* A, int M, int d, int r, bf16* const (&z)[3], int z_pitch, const Scratch& s,
                             int sm_count, int* launches, cudaStream_t st);
 // tensor_records_fit: does the context's record scratch take this call?
 bool tensor_records_fit(int M, int N, int k, const Scratch& s, int sm_count);

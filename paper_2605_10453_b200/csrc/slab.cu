@@ -510,10 +510,10 @@ static bool slab_geometry(int M, int parts, int K, int V, int k, int sm_count, b
 }
 
 // W as TMA takes it (rows of a multiple of 16 bytes; the pointer is the caller's to check), and the code likewise.
-bool slab_ok(int M, bool lowrank, int K, int V, int k, int sm_count)
+bool slab_ok(int M, int parts, int K, int V, int k, int sm_count)
 {
     SlabGeometry g;
-    return V % 8 == 0 && V >= 64 && K >= 8 && K % 8 == 0 && slab_geometry(M, lowrank ? 2 : 1, K, V, k, sm_count, false, &g);
+    return V % 8 == 0 && V >= 64 && K >= 8 && K % 8 == 0 && slab_geometry(M, parts, K, V, k, sm_count, false, &g);
 }
 
 // Any V and K, any alignment of W.

@@ -59,8 +59,7 @@ struct alignas(64) TcParams {
     unsigned long long* bound;   // mode 0: [k][bound_pitch] words (call number, key), see bound_publish
     int bound_pitch;
     unsigned int epoch;     // number of the call: larger than every earlier one's, never 0
-    bf16* z;                // mode 2: the code [M][z_pitch] and, if not null, its rounding remainder
-    bf16* z_lo;
+    bf16* z[3];             // mode 2: the code [M][z_pitch] and, if not null, its rounding remainder and what the two leave
     int z_pitch;
     int* err;
 };
@@ -511,12 +510,10 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
 #pragma unroll
             for (int q = 1; q < kTcMaxSplits; ++q)
                 if (q < p.nks) { a.x += v[q].x; a.y += v[q].y; a.z += v[q].z; a.w += v[q].w; }
-            __nv_bfloat162 h01 = __floats2bfloat162_rn(a.x, a.y), h23 = __floats2bfloat162_rn(a.z, a.w);
-            *reinterpret_cast<uint2*>(p.z + (size_t)m * p.z_pitch + col0 + c) = make_uint2(*reinterpret_cast<uint32_t*>(&h01), *reinterpret_cast<uint32_t*>(&h23));
-            if (p.z_lo != nullptr) {
-                __nv_bfloat162 l01 = __floats2bfloat162_rn(a.x - __low2float(h01), a.y - __high2float(h01));
-                __nv_bfloat162 l23 = __floats2bfloat162_rn(a.z - __low2float(h23), a.w - __high2float(h23));
-                *reinterpret_cast<uint2*>(p.z_lo + (size_t)m * p.z_pitch + col0 + c) = make_uint2(*reinterpret_cast<uint32_t*>(&l01), *reinterpret_cast<uint32_t*>(&l23));
+            for (int q = 0; q < 3 && p.z[q] != nullptr; ++q) {
+                __nv_bfloat162 h01 = __floats2bfloat162_rn(a.x, a.y), h23 = __floats2bfloat162_rn(a.z, a.w);
+                *reinterpret_cast<uint2*>(p.z[q] + (size_t)m * p.z_pitch + col0 + c) = make_uint2(*reinterpret_cast<uint32_t*>(&h01), *reinterpret_cast<uint32_t*>(&h23));
+                a.x -= __low2float(h01); a.y -= __high2float(h01); a.z -= __low2float(h23); a.w -= __high2float(h23);
             }
         }
         if (p.nks > 1) cluster_sync_exec();       // the others have read this CTA's tile
@@ -685,9 +682,9 @@ cudaError_t tensor_head(const bf16* X, const bf16* Xlo, int x_pitch, const bf16*
     return e;
 }
 
-// z = h A through the tensor cores, as bf16 [M][z_pitch] and, if z_lo is not null, its rounding remainder: the K of a tile of 128
+// z = h A through the tensor cores, as up to three bf16 matrices [M][z_pitch]: the K of a tile of 128
 // rows is split over the CTAs of a cluster, which add their partial tiles through distributed shared memory.
-cudaError_t tensor_downproj(const bf16* h, const bf16* A, int M, int d, int r, bf16* z, bf16* z_lo, int z_pitch, const Scratch& s,
+cudaError_t tensor_downproj(const bf16* h, const bf16* A, int M, int d, int r, bf16* const (&z)[3], int z_pitch, const Scratch& s,
                             int sm_count, int* launches, cudaStream_t st)
 {
     TcParams p;
@@ -711,7 +708,8 @@ cudaError_t tensor_downproj(const bf16* h, const bf16* A, int M, int d, int r, b
     p.gct = p.nct;
     p.mode = 2;
     p.k = 1;
-    p.z = z; p.z_lo = z_lo; p.z_pitch = z_pitch;
+    for (int q = 0; q < 3; ++q) p.z[q] = z[q];
+    p.z_pitch = z_pitch;
     p.err = s.err;
     // Launched early even as the first kernel of a call: apart from the weights it touches global memory only after its
     // griddepcontrol.wait, so it may come up under the tail of whatever kernel precedes it.

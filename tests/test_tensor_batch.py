@@ -88,3 +88,20 @@ def test_few_rows_matches_oracle(M, d, r, V, k, path):
     assert ctx.last_error() == binding.OK and ctx.last_path() == path
     ctx.close()
     assert check_topk(oracle.head_topk(b["h"], b["A"], b["B"], k), ids.cpu().numpy(), lp.cpu().numpy())["max_lp_err"] < 1e-4
+
+
+@pytest.mark.parametrize("M,d,r,V", [(4, 4104, 1024, 8 * 1601), (3, 512, 8192, 8 * 640), (2, 4096, 2048, 8 * 1601), (1, 2056, 2048, 8 * 1601)])
+def test_few_rows_large_A_keep_the_whole_code(M, d, r, V):
+    """One to four rows over a large A: the slab kernel, with the code in three parts, which is all of fp32."""
+    k = 10
+    ctx = binding.Context(max_M=M, max_d=max(d, r), max_V=V, max_k=k)
+    x = synth.make_inputs(M, d, r, V, seed=41)
+    g = {n: t.to(DEV) for n, t in x.items()}
+    b = {n: oracle.bf16_bits(t) for n, t in x.items()}
+    ids, lp = ctx.slimspec_head_topk(g["h"], g["A"], g["B"], k)
+    torch.cuda.synchronize()
+    assert ctx.last_error() == binding.OK and ctx.last_path() == binding.PATH_STREAM
+    ctx.close()
+    # fp32 sums of d and r products: 2^-24 sqrt(8192) = 5e-6 of a logit of at most 6; a code of 17 bits would show 1e-4 or less too,
+    # so the bound is what fp32 sums give and no more
+    assert check_topk(oracle.head_topk(b["h"], b["A"], b["B"], k), ids.cpu().numpy(), lp.cpu().numpy())["max_lp_err"] < 4e-5
