@@ -65,7 +65,7 @@ extern "C" {
 #define SLIMSPEC_PATH_AUTO 0        /* chosen per (M, shapes) from measured timings            */
 #define SLIMSPEC_PATH_GENERIC 1     /* any shape.  Forced: one thread per logit, slow.  Chosen by AUTO:
                                        the streaming tensor-core kernel, up to 64 rows a launch */
-#define SLIMSPEC_PATH_STREAM 2      /* split-V weight-streaming kernels (M <= 16 per launch)   */
+#define SLIMSPEC_PATH_STREAM 2      /* split-V weight-streaming kernels (M <= 64 per launch)   */
 #define SLIMSPEC_PATH_TENSOR 3      /* tcgen05 / TMEM tensor-core kernels (large M)            */
 
 typedef struct slimspec_ctx slimspec_ctx;

@@ -86,18 +86,26 @@ def strerror(status: int) -> str:
     return load().slimspec_strerror(int(status)).decode()
 
 
+# A small head runs for as long as the interpreter takes to marshal its call (about 10 us), so the steps that
+# every call repeats are kept few: plain integers for pointers (argtypes converts them), no Stream object for the
+# current stream, shapes compared as they are.
 def _ptr(t):
-    return None if t is None else ctypes.c_void_p(t.data_ptr())
+    return None if t is None else t.data_ptr()
+
+
+_raw_stream = getattr(torch._C, "_cuda_getCurrentRawStream", None)
 
 
 def _stream(stream):
-    if stream is None:
-        stream = torch.cuda.current_stream()
-    return ctypes.c_void_p(stream.cuda_stream)
+    if stream is not None:
+        return stream.cuda_stream
+    if _raw_stream is not None:
+        return _raw_stream(torch.cuda.current_device())
+    return torch.cuda.current_stream().cuda_stream
 
 
 def _check_dev(t, dtype, shape, name):
-    if not t.is_cuda or t.dtype != dtype or tuple(t.shape) != tuple(shape) or not t.is_contiguous():
+    if not t.is_cuda or t.dtype != dtype or t.shape != shape or not t.is_contiguous():
         raise ValueError("%s must be a contiguous CUDA %s tensor of shape %s" % (name, dtype, tuple(shape)))
 
 

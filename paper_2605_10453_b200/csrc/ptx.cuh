@@ -55,26 +55,9 @@ __device__ __forceinline__ bool mbar_try_wait(uint64_t* bar, uint32_t parity)
     return ok != 0;
 }
 
-// Wait for the phase with the given parity.  Gives up when the spin budget is spent or
-// another thread of the CTA has already given up (*abort != 0); on giving up it records
-// `code` in the global error word and raises the CTA's abort flag.  Returns success.
-__device__ __forceinline__ bool mbar_wait(uint64_t* bar, uint32_t parity, volatile int* abort, int* err, int code)
-{
-    for (uint32_t it = 0; it < kSpinLimit; ++it) {
-        if (mbar_try_wait(bar, parity)) return true;
-        if (it > 1024) {
-            if (*abort) return false;
-            __nanosleep(64);
-        }
-    }
-    *abort = 1;
-    atomicCAS(err, 0, code);
-    return false;
-}
-
-// The same for a whole converged warp: lane 0 polls, sleeping between polls, and the result is
-// shared.  Thirty-two lanes polling per waiting warp kept the shared-memory pipe busy enough to
-// slow the thread that issues the tensor-core instructions.
+// Wait of a whole converged warp for the phase with the given parity: lane 0 polls, sleeping between polls, and the result is
+// shared.  Gives up when the spin budget is spent or another thread of the CTA has already given up (*abort != 0); on giving
+// up it records `code` in the global error word and raises the CTA's abort flag.  Returns success.
 __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, volatile int* abort, int* err, int code)
 {
     int ok = 1;
@@ -98,7 +81,7 @@ __device__ __forceinline__ bool mbar_wait_warp(uint64_t* bar, uint32_t parity, v
 // The same for a converged warp that issues tensor-core or TMA instructions, where the time of a wait that is over already
 // counts.  The loop is one asm statement and the result a vote: the compiler then keeps what is the same in all lanes in uniform
 // registers across the wait.  (Cycles per 128 x 64 x 16 MMA, one such wait and a commit per four: no wait 48, this 63,
-// a C++ loop over mbar_try_wait 86, mbar_wait 92.)  A warp that stops for a wait that ran out reports it by mbar_gave_up.
+// a C++ loop over mbar_try_wait 86, one with its slow path inlined 92.)  A warp that stops for a wait that ran out reports it by mbar_gave_up.
 __device__ __forceinline__ bool mbar_wait_uniform(uint64_t* bar, uint32_t parity)
 {
     uint32_t ok;
@@ -114,7 +97,7 @@ __device__ __forceinline__ bool mbar_wait_uniform(uint64_t* bar, uint32_t parity
         "DONE:\n\t"
         "selp.u32 %0, 1, 0, p;\n\t}"
         : "=r"(ok)
-        : "r"(smem_u32(bar)), "r"(parity), "n"(kSpinLimit)
+        : "r"(smem_u32(bar)), "r"(parity), "n"(kSpinLimit / 4)
         : "memory");
     return __all_sync(0xffffffffu, ok != 0u);
 }
@@ -250,12 +233,6 @@ __device__ __forceinline__ void tma_load_2d_pair(void* dst, const void* tensor_m
             smem_u32(dst)),
         "l"(tensor_map), "r"(x), "r"(y), "r"(bar)
         : "memory");
-}
-
-// The box's lines are brought into the L2.
-__device__ __forceinline__ void tma_prefetch_2d(const void* tensor_map, int x, int y)
-{
-    asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(tensor_map), "r"(x), "r"(y) : "memory");
 }
 
 // ---- tcgen05: tensor memory, MMA issue, completion, loads

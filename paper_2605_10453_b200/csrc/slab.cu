@@ -353,6 +353,7 @@ __global__ void __maxnreg__(RAGGED ? 96 : 112) k_slab_head(const __grid_constant
         int s = 0, ph = 0;
         uint32_t st = ring_w;
         bool alive = true;
+        pdl_wait();          // nothing to do before the code is there, and the waits below are bounded
         for (int i = 0; i < p.nst; ++i) {
             if (alive) alive = mbar_wait_uniform(&full[s], ph);
             if (alive) {
@@ -406,8 +407,8 @@ __global__ void __maxnreg__(RAGGED ? 96 : 112) k_slab_head(const __grid_constant
     }
 
     // ================= tail: all warps.  Everything below writes what belongs to the kernels ahead in the stream.
+    pdl_wait();          // before the bounded wait: what the kernels ahead take is not this one's
     const bool ok = mbar_wait_warp(&acc_full, 0, abort_flag, p.err, ERR_WAIT_ACC);
-    pdl_wait();
     tc_fence_after_sync();
     float* lg = reinterpret_cast<float*>(ring);          // the ring is idle: every stage has been multiplied
     unsigned char* row_area = reinterpret_cast<unsigned char*>(lg + (size_t)RG * p.lpitch) + warp * kSlabRowBytes;

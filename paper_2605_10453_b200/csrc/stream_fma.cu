@@ -11,7 +11,7 @@
 // leave the SM: each CTA writes max / sum-exp / top-k of its slab as a record and the last CTA to
 // arrive merges the records (Section 4.1: both projections; the softmax of Section 3.2 in online
 // form; the candidate selection).
-// (Three to sixteen rows take the tensor-core streaming kernel of stream.cu.)
+// (More rows, and these over a very large A, take the slab kernel.)
 #include "kernels.h"
 #include "ptx.cuh"
 #include "select.cuh"

@@ -315,6 +315,7 @@ __global__ void __launch_bounds__(kTcThreads, 1) k_tc_gemm(const __grid_constant
             int s = 0, ph = 0;
             uint32_t st = ring_w;
             bool alive = true;
+            pdl_wait();          // nothing to do before X is there, and the waits below are bounded
             for (int t = 0; t < ntiles; ++t) {
                 const int buf = t & 1;
                 if (t >= 2 && alive) alive = mbar_wait_uniform(&acc_empty[buf], ((t >> 1) - 1) & 1);
